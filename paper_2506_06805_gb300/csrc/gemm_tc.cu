@@ -278,7 +278,7 @@ struct alignas(64) TcProblem {
 // Epilogue write modes. The FP64 pipe of this GPU retires about two
 // operations per SM clock, so the per-element path tests integers only.
 enum { WM_F32 = 0, WM_F64_ADD = 1, WM_F64_STORE = 2, WM_F64_BETA = 3 };
-constexpr int MAX_PROBLEMS = 16;
+constexpr int MAX_PROBLEMS = TC_MAX_PROBLEMS;
 struct TcGroup {
   TcProblem p[MAX_PROBLEMS];
   int nprob;
@@ -1026,28 +1026,31 @@ Choice tune(const TcDesc &g, cudaStream_t st, int *err) {
 
 }  // namespace
 
+void gemm_tc_tune(TcDesc *g, cudaStream_t st, int *err) {
+  if (!(tune_enabled() || tune_path())) return;
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  tune_load();
+  const std::string key = tune_key(*g);
+  auto it = g_tune.find(key);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(st, &cap);
+  if (it == g_tune.end() && tune_enabled() && !g->no_tune && cap == cudaStreamCaptureStatusNone) {
+    g_tune[key] = tune(*g, st, err);
+    tune_save();
+    it = g_tune.find(key);
+  }
+  if (it != g_tune.end()) {
+    g->bn = it->second.bn;
+    g->group_m = it->second.group_m;
+    g->chunk = it->second.chunk;
+  }
+}
+
 void gemm_tc(const TcDesc &g0, cudaStream_t st, int *err) {
   if (g0.M <= 0 || g0.N <= 0 || g0.Kp <= 0) return;
   check_desc(g0);
   TcDesc g = g0;
-  if (tune_enabled() || tune_path()) {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    tune_load();
-    const std::string key = tune_key(g);
-    auto it = g_tune.find(key);
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(st, &cap);
-    if (it == g_tune.end() && tune_enabled() && !g.no_tune && cap == cudaStreamCaptureStatusNone) {
-      g_tune[key] = tune(g, st, err);
-      tune_save();
-      it = g_tune.find(key);
-    }
-    if (it != g_tune.end()) {
-      g.bn = it->second.bn;
-      g.group_m = it->second.group_m;
-      g.chunk = it->second.chunk;
-    }
-  }
+  gemm_tc_tune(&g, st, err);
   const bool wide = g.bn > 0 ? g.bn == 256 : g.N >= 192;
   dispatch(&g, 1, wide, st, err);
 }

@@ -89,9 +89,14 @@ struct TcDesc {
   bool no_tune = false;
 };
 void gemm_tc(const TcDesc &g, cudaStream_t st, int *err_flag);
+// Tile choices of the autotuner for g's shape bucket, when it is on or has a
+// saved choice (gemm_tc does this by itself): sets bn, group_m and chunk.
+void gemm_tc_tune(TcDesc *g, cudaStream_t st, int *err_flag);
+// Problems one grouped launch takes at most.
+constexpr int TC_MAX_PROBLEMS = 16;
 // Several independent GEMMs (any shapes, same or mixed tiers) in as few
-// persistent launches as possible: one per tier and tile width, up to 16
-// problems each, sharing one tile queue.
+// persistent launches as possible: one per tier and tile width, up to
+// TC_MAX_PROBLEMS problems each, sharing one tile queue.
 void gemm_tc_grouped(const std::vector<TcDesc> &descs, cudaStream_t st, int *err_flag);
 // Padded K granularity (real elements) for a tier: 32 for tf32, 64 for bf16.
 // Tile width for N columns: 256 unless 128-wide tiles waste clearly less
