@@ -27,6 +27,7 @@
 #include <cuda_fp16.h>
 
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -741,11 +742,21 @@ void launch(const TcDesc *descs, int n, cudaStream_t st, int *err) {
     a.k_splits = (a.num_kb + a.kb_per_split - 1) / a.kb_per_split;
     a.m_tiles = static_cast<int>((mr + UNIT_ROWS - 1) / UNIT_ROWS);
     a.n_tiles = static_cast<int>((g.N + BN - 1) / BN);
-    // raster groups: as many A panels (a unit's rows x the K range of a
-    // split) as fit in ~24 MB of L2 share each B panel while it is resident
+    // raster groups of m tiles (n swept inside a group). As many A panels (a
+    // unit's rows x the K range of a split) as fit in ~24 MB of L2 share each
+    // B panel while it is resident. A long K leaves room for one panel or
+    // none; what counts then is the set of tiles in flight, which stream
+    // their panels along K together: with g m tiles and P / g n tiles among
+    // the P resident units, the rows read per K block are least at
+    // g = sqrt(P BN / UNIT_ROWS). With one group per panel the o^3 v^3 ring
+    // product at o = 40, v = 300 (K = 24000) read 49 GB from DRAM in 9.4 ms;
+    // the FP16 residual at that size takes 103.8 ms instead of 105.2 with
+    // this rule.
     const double panel = static_cast<double>(UNIT_ROWS) * a.kb_per_split * ROW_BYTES * (SPLIT ? 2 : 1);
+    const double square = std::sqrt(static_cast<double>(PAIR ? sms / 2 : sms) * BN / UNIT_ROWS);
     a.group_m = g.group_m > 0 ? std::min(g.group_m, a.m_tiles)
-                              : static_cast<int>(std::max(1.0, std::min<double>(a.m_tiles, 24.0e6 / panel)));
+                              : static_cast<int>(std::min<double>(a.m_tiles, std::max(square, 24.0e6 / panel)));
+    a.group_m = std::max(a.group_m, 1);
     a.chunk = g.chunk > 0 ? g.chunk : default_chunk(g.tier, a.kb_per_split);
     a.out = g.out;
     a.wmode = g.out == TC_OUT_F32 ? WM_F32
