@@ -373,7 +373,9 @@ bool Engine::run(cplx alpha, const TRef &A, const TRef &B, cplx beta, const TRef
   if (mdim.empty()) { lda = 0; ldc = 0; }
   if (ndim.empty()) ldb = 0;
 
-  // small or skinny products stay on the CUDA-core path (GEMV or a few tiles)
+  // small or skinny products stay on the CUDA-core path (GEMV or a few
+  // tiles); FP64 products large enough for it run on the tensor cores, exact
+  // to FP64
   if (simt) {
     GemmDesc g;
     g.M = M; g.N = N; g.K = K;
@@ -383,7 +385,11 @@ bool Engine::run(cplx alpha, const TRef &A, const TRef &B, cplx beta, const TRef
     g.alpha = alpha; g.beta = beta;
     g.k_contig = kdim.empty() || (M == 1 ? bkstr.back() == 1 : akstr.back() == 1);
     g.f32 = tier != TIER_FP64;
-    gemm_f64(g, st, num_sms);
+    if (tier == TIER_SIMT32)
+      gemm_f64(g, st, num_sms);
+    else
+      product_f64(g, !mdim.empty() && amstr.back() == 1 && !kdim.empty() && akstr.back() != 1,
+                  !ndim.empty() && bnstr.back() == 1 && !kdim.empty() && bkstr.back() != 1);
     return false;
   }
   // short contracted index with one short free side: FP32 on the CUDA cores
@@ -491,6 +497,98 @@ bool Engine::run(cplx alpha, const TRef &A, const TRef &B, cplx beta, const TRef
   Region r = region("gemm " + A.idx + "," + B.idx + "->" + C.idx);
   gemm_tc(t, st, err_flag);
   return false;
+}
+
+void Engine::product_f64(const GemmDesc &g, bool a_rows, bool b_rows) {
+  if (slices_pay(g.M, g.N, g.K) && run_slices(g, a_rows, b_rows)) return;
+  gemm_f64(g, st, num_sms);
+}
+
+size_t Engine::slice_budget(int which) {
+  const auto it = planes_.find(which);
+  const size_t held = it == planes_.end() ? 0 : it->second.bytes;
+  return std::max(held, std::min(SLICE_BUDGET, device_avail(al) / 8));
+}
+
+bool Engine::run_slices(const GemmDesc &g, bool a_rows, bool b_rows) {
+  // a capped context keeps the memory its cap was chosen for
+  if (al->limit) return false;
+  const size_t cap_a = slice_budget(SLICE_SLOT_A), cap_b = slice_budget(SLICE_SLOT_B);
+  // K blocks keep the integer sums of a tile within their range
+  const long kb = std::min<long>(g.K, 65536);
+  auto rows_in = [&](bool a_side, size_t cap, long rows) {
+    if (slice_bytes(a_side, rows, kb) <= cap) return rows;
+    const size_t per = slice_bytes(a_side, 1024, kb) / 1024 + 1;
+    return static_cast<long>(cap / per) / 256 * 256;
+  };
+  // (4.1 M rows: the guarded FP64 launch's grid)
+  const long mb = std::min<long>(rows_in(true, cap_a, g.M), 4000000);
+  const long nb = rows_in(false, cap_b, g.N);
+  if (mb < std::min<long>(g.M, 256) || nb < std::min<long>(g.N, 256)) return false;
+  void *ma, *mbuf;
+  try {
+    ma = plane(SLICE_SLOT_A, slice_bytes(true, mb, kb));
+    mbuf = plane(SLICE_SLOT_B, slice_bytes(false, nb, kb));
+  } catch (const Error &e) {
+    if (e.code != CC_ERR_OOM) throw;
+    ++gen;  // a plane may have been given up
+    return false;
+  }
+  auto at = [](const cplx *p, const long *&t, long i0, long ld) {
+    if (t) t += i0;
+    return t ? p : p + i0 * ld;
+  };
+  for (long k0 = 0; k0 < g.K; k0 += kb) {
+    const long K = std::min(kb, g.K - k0);
+    for (long n0 = 0; n0 < g.N; n0 += nb) {
+      const long N = std::min(nb, g.N - n0);
+      SliceGemm s;
+      s.N = N;
+      s.B = slice_planes(mbuf, false, N, K);
+      SliceOperand ob;
+      ob.rt = g.bn;
+      ob.kt = g.bk;
+      ob.src = at(at(g.B, ob.rt, n0, g.ldb), ob.kt, k0, 1);
+      ob.ld = g.ldb;
+      ob.rows = N;
+      ob.conj = g.conjB;
+      ob.rows_unit = b_rows;
+      for (long m0 = 0; m0 < g.M; m0 += mb) {
+        const long M = std::min(mb, g.M - m0);
+        s.M = M;
+        s.A = slice_planes(ma, true, M, K);
+        SliceOperand oa;
+        oa.rt = g.am;
+        oa.kt = g.ak;
+        oa.src = at(at(g.A, oa.rt, m0, g.lda), oa.kt, k0, 1);
+        oa.ld = g.lda;
+        oa.rows = M;
+        oa.conj = g.conjA;
+        oa.rows_unit = a_rows;
+        {
+          Region r = region("slice pack");
+          slice_pack(&oa, &s.A, m0 == 0 ? &ob : nullptr, &s.B, K, st, num_sms);
+        }
+        s.cm = g.cm;
+        s.cn = g.cn;
+        s.ldc = g.ldc;
+        s.C = const_cast<cplx *>(at(at(g.C, s.cm, m0, g.ldc), s.cn, n0, 1));
+        s.alpha = g.alpha;
+        s.beta = k0 == 0 ? g.beta : C1();
+        s.src = g;
+        s.src.K = K;
+        s.src.A = oa.src;
+        s.src.am = oa.rt;
+        s.src.ak = oa.kt;
+        s.src.B = ob.src;
+        s.src.bn = ob.rt;
+        s.src.bk = ob.kt;
+        Region r = region("slice gemm");
+        gemm_slices(s, st, err_flag, num_sms);
+      }
+    }
+  }
+  return true;
 }
 
 void Engine::permute_into(cplx alpha, const TRef &in, cplx beta, const TRef &out) {

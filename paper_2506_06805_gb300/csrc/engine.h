@@ -97,6 +97,19 @@ class Engine {
   const long *table(const std::vector<long> &dims, const std::vector<long> &strides);
   // growable scratch planes for the tensor-core operands
   void *plane(int which, size_t bytes);
+  // FP64 product of g: on the tensor cores where that pays (gemm_slices.cu),
+  // else on the FP64 pipe. a_rows, b_rows: neighbouring rows of the operand
+  // are neighbours in memory and k is strided.
+  void product_f64(const GemmDesc &g, bool a_rows, bool b_rows);
+  // The tensor-core form in blocks of rows, columns and K that fit the plane
+  // budget; false (nothing done) when there is no room for planes worth having
+  bool run_slices(const GemmDesc &g, bool a_rows, bool b_rows);
+  // Device bytes each operand's digit planes of an FP64 product may take:
+  // what is already held in their slot, or up to an eighth of the room left
+  // and SLICE_BUDGET
+  size_t slice_budget(int which);
+  static constexpr size_t SLICE_BUDGET = size_t(4) << 30;
+  static constexpr int SLICE_SLOT_A = 1000, SLICE_SLOT_B = 1001;
   void clear_cache() {
     cache_.clear();
     packs_.clear();

@@ -29,6 +29,47 @@ struct GemmDesc {
 // FP64 SIMT path (CC_TIER_FP64).
 void gemm_f64(const GemmDesc &g, cudaStream_t st, int num_sms);
 
+// The plain tiled FP64 kernel of g, computed only if *flag_a or *flag_b is
+// nonzero on the device (otherwise the launch returns at once).
+void gemm_f64_if(const GemmDesc &g, const int *flag_a, const int *flag_b, cudaStream_t st);
+
+// FP64 products on the tensor cores (gemm_slices.cu): operands cut into
+// SLICE_COUNT planes of integer digits relative to each row's largest
+// magnitude, products of the planes summed exactly.
+constexpr int SLICE_COUNT = 7;
+struct SliceOperand {  // rows x K source elements, addressed as in GemmDesc
+  const cplx *src = nullptr;
+  const long *rt = nullptr, *kt = nullptr;
+  long ld = 0;
+  long rows = 0;
+  bool conj = false;
+  bool rows_unit = false;  // neighbouring rows are neighbours in memory, k is strided
+};
+struct SlicePlanes {
+  void *planes = nullptr;  // [SLICE_COUNT][plane_rows][Kp] FP16
+  int *e = nullptr;        // [rows] exponents, then the Inf/NaN flag
+  float *n2 = nullptr;     // [rows] squared 2-norms relative to the row's 2^E
+  long rows = 0, plane_rows = 0, Kp = 0;
+};
+long slice_kp(long K);
+// bytes of an operand's planes and exponents (A side: rows expanded by two)
+size_t slice_bytes(bool a_side, long rows, long K);
+SlicePlanes slice_planes(void *mem, bool a_side, long rows, long K);  // views into slice_bytes() bytes
+// planes of one or both operands (either side may be NULL)
+void slice_pack(const SliceOperand *A, const SlicePlanes *pa, const SliceOperand *B,
+                const SlicePlanes *pb, long K, cudaStream_t st, int num_sms);
+struct SliceGemm {
+  long M = 0, N = 0;             // complex rows a_row0 .. of A, rows b_row0 .. of B
+  SlicePlanes A, B;
+  long a_row0 = 0, b_row0 = 0;
+  cplx *C = nullptr; const long *cm = nullptr, *cn = nullptr; long ldc = 0;
+  cplx alpha = {1.0, 0.0}, beta = {0.0, 0.0};
+  GemmDesc src;                  // the operands themselves (A, B, K and their addressing)
+};
+void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err_flag, int num_sms);
+// whether an M x N x K FP64 product is expected to be faster this way
+bool slices_pay(long M, long N, long K);
+
 // Skinny complex product on the CUDA cores:
 //   C[cb(r) + cs(s)] = alpha sum_k G[r][k] S[s][k] + beta C
 // for r < Mb (long side), s < Ns (short side), k < K. Row offsets are

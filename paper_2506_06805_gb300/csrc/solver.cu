@@ -540,14 +540,20 @@ namespace {
 // FP16x3 ladder at o = 23, v = 187, X = 748 14.06 -> 10.85 ms; FP16 residual
 // at o = 20, v = 160, X = 640 8.29 -> 7.39 ms, at o = 40, v = 300, X = 1200
 // 107.8 -> 105.2 ms. The values of the computed elements do not change.
-std::vector<std::pair<long, long>> slab_rows(long v, long a0, long nA) {
-  auto units = [&](long s0, long s1) {
-    return ((2 * (s1 - s0) * v + 255) / 256) * (((v - s0 - 1) * v + 255) / 256);
+//
+// f64_aux != 0: one FP64 launch per range over f64_aux auxiliary indices, so a
+// range costs whole waves of the 76 CTA pairs (K blocks of 32 complex, three
+// for a tile's epilogue) and a launch (two K blocks' time).
+std::vector<std::pair<long, long>> slab_rows(long v, long a0, long nA, long f64_aux = 0) {
+  auto cost = [&](long s0, long s1) {
+    const long m = (2 * (s1 - s0) * v + 255) / 256;
+    if (!f64_aux) return m * (((v - s0 - 1) * v + 255) / 256);
+    return (m * (((v - s0 - 1) * v + 127) / 128) + 75) / 76 * ((f64_aux + 31) / 32 + 3) + 2;
   };
   long best = -1, best_n = 1;
   for (long n = 1; n <= std::min<long>(TC_MAX_PROBLEMS, nA); ++n) {
     long u = 0;
-    for (long q = 0; q < n; ++q) u += units(a0 + nA * q / n, a0 + nA * (q + 1) / n);
+    for (long q = 0; q < n; ++q) u += cost(a0 + nA * q / n, a0 + nA * (q + 1) / n);
     if (best < 0 || u < best) {
       best = u;
       best_n = n;
@@ -594,9 +600,23 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
   const size_t veb = fast ? sizeof(float2) : sizeof(cplx);
 
   if (!fast) {
-    // K-major copy of L: LT[(a,c)][P]
-    Buf LT(&al, sizeof(cplx) * vv * X);
-    eng.permute_into(C1(), T(Lv, "Pac", {X, v, v}), C0(), T(LT.c(), "acP", {v, v, X}));
+    // L's digit planes are made once when they fit, rows (a, c) read along c;
+    // otherwise each product makes its own from a K-major copy LT[(a,c)][P]
+    Buf LT, LA, LB;
+    SlicePlanes pA, pB;
+    if (al.limit == 0 && X <= 65536 && slices_pay(v, vv, X) &&
+        slice_bytes(true, vv, X) <= std::min(Engine::SLICE_BUDGET, device_avail(&al) / 8)) {
+      LA.reset(&al, slice_bytes(true, vv, X));
+      LB.reset(&al, slice_bytes(false, vv, X));
+      pA = slice_planes(LA.p, true, vv, X);
+      pB = slice_planes(LB.p, false, vv, X);
+      SliceOperand l;
+      l.src = Lv; l.kt = ptab; l.ld = 1; l.rows = vv; l.rows_unit = true;
+      slice_pack(&l, &pA, &l, &pB, X, st, num_sms);
+    } else {
+      LT.reset(&al, sizeof(cplx) * vv * X);
+      eng.permute_into(C1(), T(Lv, "Pac", {X, v, v}), C0(), T(LT.c(), "acP", {v, v, X}));
+    }
     long a0 = 0;
     Buf Vs, W;
     while (a0 < v - 1) {
@@ -609,12 +629,26 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
       const long np = p1 - p0;
       B(Vs, nA * per_a);
       B(W, np * n_cd);
-      GemmDesc g1;
-      g1.M = nA * v; g1.N = (v - a0) * v; g1.K = X;
-      g1.A = LT.c() + a0 * v * X; g1.lda = X;
-      g1.B = LT.c() + a0 * v * X; g1.ldb = X;
-      g1.C = Vs.c(); g1.ldc = (v - a0) * v;
-      gemm_f64(g1, st, num_sms);
+      for (const auto &ar : slab_rows(v, a0, nA, X)) {
+        const long s0 = ar.first, s1 = ar.second;
+        GemmDesc g1;
+        g1.M = (s1 - s0) * v; g1.N = (v - s0 - 1) * v; g1.K = X;
+        g1.C = Vs.c() + (s0 - a0) * v * (v - a0) * v + (s0 + 1 - a0) * v; g1.ldc = (v - a0) * v;
+        if (LA.p) {
+          g1.A = Lv + s0 * v; g1.lda = 1; g1.ak = ptab;
+          g1.B = Lv + (s0 + 1) * v; g1.ldb = 1; g1.bk = ptab;
+          SliceGemm sg;
+          sg.M = g1.M; sg.N = g1.N; sg.A = pA; sg.B = pB;
+          sg.a_row0 = s0 * v; sg.b_row0 = (s0 + 1) * v;
+          sg.C = g1.C; sg.ldc = g1.ldc;
+          sg.src = g1;
+          gemm_slices(sg, st, err_d.as<int>(), num_sms);
+        } else {
+          g1.A = LT.c() + s0 * v * X; g1.lda = X;
+          g1.B = LT.c() + (s0 + 1) * v * X; g1.ldb = X;
+          eng.product_f64(g1, false, false);
+        }
+      }
       ladder_antisym(Vs.p, false, v, static_cast<int>(a0), static_cast<int>(nA), p0, p1,
                      ab_a.as<int>(), ab_b.as<int>(), ab_a.as<int>(), ab_b.as<int>(), TIER_FP64,
                      nullptr, nullptr, 0, W.c(), st);
@@ -623,7 +657,7 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
       g2.A = tau; g2.am = rt.as<long>(); g2.ak = kt.as<long>();
       g2.B = W.c(); g2.ldb = n_cd;
       g2.C = Rp.c() + p0; g2.ldc = n_ab;
-      gemm_f64(g2, st, num_sms);
+      eng.product_f64(g2, false, false);
       a0 = a1;
     }
   } else {
@@ -936,7 +970,12 @@ void Ctx::residual(const cplx *t1p, const cplx *t2p, cplx *R1, cplx *R2) {
 // CCSD iterations with Jacobi updates and DIIS
 // ===========================================================================
 size_t Ctx::planes_bytes_estimate(int tr) const {
-  if (tr == TIER_FP64) return 0;
+  if (tr == TIER_FP64) {
+    // digit planes of the largest product, as far as the budget goes
+    const double mkk = static_cast<double>(o) * o * v * v * 2.0 * SLICE_COUNT;
+    const double cap = 1.125 * static_cast<double>(Engine::SLICE_BUDGET);
+    return al.limit ? 0 : static_cast<size_t>(std::min(cap, 4.0 * mkk) + std::min(cap, 2.0 * mkk));
+  }
   // the largest doubles-sized contraction (M K = o^2 v^2, N <= M) packs its
   // A side into 2M x 2K and its B side into N x 2K elements of the tier's
   // type, twice for the hi/lo tiers

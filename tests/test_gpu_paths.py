@@ -45,3 +45,104 @@ def test_ladder_row_ranges(tier, o, v, slab):
         s.ladder_dev(torch.from_numpy(tau).cuda(), out)
     err = np.abs(out.cpu().numpy() - ref).max() / np.abs(ref).max()
     assert err <= LADDER_TOL[tier]
+
+
+def _cn(g, *shape):
+    return torch.view_as_complex(torch.randn(*shape, 2, generator=g, device="cuda", dtype=torch.float64))
+
+
+def _rownorm(x):
+    """Row 2-norms without under- or overflow."""
+    top = x.abs().amax(1)
+    scaled = torch.view_as_real(x).flatten(1) / torch.where(top == 0, 1.0, top)[:, None]
+    return torch.linalg.vector_norm(scaled, dim=1) * top
+
+
+def _check_product(A, B, C):
+    """Both sides are FP64 sums of K terms: sqrt(K) 2^-52 of |a_m| |b_n|."""
+    ref = A @ B.T
+    tol = A.shape[1] ** 0.5 * 2.0 ** -52 * _rownorm(A)[:, None] * _rownorm(B)[None, :]
+    assert bool(((C - ref).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("M,N,K", [(257, 129, 300), (129, 2000, 33), (64, 640, 1025), (5, 40000, 160),
+                                   (700, 700, 64), (300, 130, 40000), (130, 130, 65537),
+                                   (1200, 64, 65600), (64, 2500, 65600)])
+def test_fp64_product_on_tensor_cores(M, N, K):
+    """Ragged tiles, few rows, a split K, K in two blocks, and operands whose
+    digit planes exceed the plane budget (the last two, blocked in M and N)."""
+    P = _gpu()
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A, B = _cn(g, M, K), _cn(g, N, K)
+    C = torch.empty((M, N), dtype=torch.complex128, device="cuda")
+    P.zgemm_dev(A, B, C, "fp64")
+    _check_product(A, B, C)
+
+
+def test_fp64_product_extreme_rows():
+    """Rows of any scale (to the smallest denormals), zero rows, rows with one
+    large element, and Inf / NaN, which the tensor-core form leaves to the
+    FP64 kernel."""
+    P = _gpu()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    M, N, K = 300, 260, 500
+    A, B = _cn(g, M, K), _cn(g, N, K)
+    A[1] = 0
+    A[2] *= 1e-310
+    A[3] *= 1e280
+    B[3] *= 1e-280
+    A[4] *= 1e150
+    B[4] *= 1e150
+    A[5, 7] *= 1e12
+    B[6] = 0.5 + 0.5j
+    A[6] = 1.0
+    C = torch.empty((M, N), dtype=torch.complex128, device="cuda")
+    P.zgemm_dev(A, B, C, "fp64")
+    ref = A @ B.T
+    tol = K ** 0.5 * 2.0 ** -52 * _rownorm(A)[:, None] * _rownorm(B)[None, :]
+    ok = (C - ref).abs() <= tol + 1e-321  # the products of row 2 are themselves denormal
+    ok[3, 4] = not bool(torch.isfinite(C[3, 4]))  # 1e430
+    assert bool(ok.all())
+    assert bool((C[1] == 0).all())
+    for bad in (float("inf"), float("nan")):
+        A2 = A.clone()
+        A2[10, 20] = bad
+        P.zgemm_dev(A2, B, C, "fp64")
+        keep = torch.arange(M, device="cuda") != 10
+        ok = (C - ref).abs() <= tol + 1e-321
+        ok[3, 4] = True
+        assert bool(ok[keep].all())
+        assert not bool(torch.isfinite(torch.view_as_real(C[10])).any(-1).any())
+
+
+@pytest.mark.parametrize("o,v,X", [(6, 41, 163), (9, 30, 121)])
+def test_fp64_residual_and_sigma_on_tensor_cores(o, v, X):
+    """Strided, conjugated, transposed and accumulating products of the FP64
+    residual and sigma at sizes that take the tensor-core form."""
+    from oracle import ipeom
+    P = _gpu()
+    eps, L = synth.make_system(o, v, X, seed=5)
+    L = 4 * L
+    rng = np.random.default_rng(2)
+    t1 = 0.02 * (rng.standard_normal((o, v)) + 1j * rng.standard_normal((o, v)))
+    t2 = _amps(rng, o, v)
+    g = integrals.blocks_from_cholesky(L, o)
+    R1, R2 = ccsd.residuals(g, eps, t1, t2)
+    io, jo = np.triu_indices(o, 1)
+    av, bv = np.triu_indices(v, 1)
+    d1, d2 = torch.from_numpy(t1).cuda(), torch.from_numpy(t2).cuda()
+    r1, r2 = torch.empty_like(d1), torch.empty_like(d2)
+    with P.System(eps, L, n_occ=o, tier="fp64") as s:
+        s.residual_dev(d1, d2, r1, r2)
+        s.set_amplitudes(t1, t2[io, jo][:, av, bv])
+        H = ipeom.hbar(g, eps, t1, t2)
+        n = ipeom.dim(o, v)
+        x = rng.standard_normal((7, n)) + 1j * rng.standard_normal((7, n))
+        xd = torch.from_numpy(x).cuda()
+        sd, ld = torch.empty_like(xd), torch.empty_like(xd)
+        s.sigma_dev(xd, sd)
+        s.left_sigma_dev(xd, ld)
+    for got, ref in ((r1, R1), (r2, R2),
+                     (sd, np.array([ipeom.sigma(H, x[k], o, v) for k in range(7)])),
+                     (ld, np.array([ipeom.left_sigma(H, x[k], o, v) for k in range(7)]))):
+        assert np.abs(got.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
