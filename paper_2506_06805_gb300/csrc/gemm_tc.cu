@@ -181,6 +181,8 @@ __global__ void __launch_bounds__(320, 1)
     if (lane == 0) {
       // ---------------- TMA producer ----------------
       long it = 0;  // k blocks issued so far (all tiles)
+      int s = 0;    // their stage, and the parity of the wait for it to be free
+      uint32_t ph = 1;
       bool ok = true;
       for (int t = TC_UNIT0; t < n_units && ok; t += TC_USTEP) {
         const TcProblem &P = grp.p[find_problem(grp, t)];
@@ -191,9 +193,7 @@ __global__ void __launch_bounds__(320, 1)
         const int ya = m_tile * UNIT_ROWS + TC_RANK * BM;
         const int yb = PAIR ? n_tile * BN + TC_RANK * (BN / 2) : n_tile * BN;
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = static_cast<int>(it % STAGES);
-          const uint32_t ph = static_cast<uint32_t>(it / STAGES) & 1u;
-          if (!mbar_wait(&empty[s], ph ^ 1u, wait_ns)) {
+          if (!mbar_wait(&empty[s], ph, wait_ns)) {
             atomicExch(err, 1);
             ok = false;
             break;
@@ -218,6 +218,10 @@ __global__ void __launch_bounds__(320, 1)
               tma_load_2d(st + 2 * A_BYTES + B_BYTES, &P.mBlo, &full[s], kx, yb);
             }
           }
+          if (++s == STAGES) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
       }
       // the last load issued into each stage must land before the CTA exits
@@ -232,11 +236,18 @@ __global__ void __launch_bounds__(320, 1)
       }
     }
   } else if (warp == 9) {
-    if (lane == 0 && TC_RANK == 0) {
+    if (TC_RANK == 0 && elect_one()) {
       // ---------------- MMA issuer (the leader of a pair) ----------------
-      long it = 0;  // k blocks consumed (all tiles)
+      // One thread feeds the tensor core, so its instructions per K block
+      // count: an elected lane, running stage counters and descriptors that
+      // differ by added offsets (FP16x3 ladder at o = 23, v = 187, X = 748
+      // 10.85 -> 10.71 ms, FP16 residual at o = 20, v = 160, X = 640 7.38 ->
+      // 7.26 ms, at o = 40, v = 300, X = 1200 103.8 -> 102.8 ms).
+      int s = 0;    // stage of the next k block, and its parity
+      uint32_t ph = 0;
       long c = 0;   // chunks issued (all tiles)
       bool ok = true;
+      const uint64_t desc0 = sw128_desc(smem_u32(smem));
       for (int t = TC_UNIT0; t < n_units && ok; t += TC_USTEP) {
         const TcProblem &P = grp.p[find_problem(grp, t)];
         int m_tile, n_tile, z;
@@ -255,30 +266,31 @@ __global__ void __launch_bounds__(320, 1)
           tc_fence_after();
           const uint32_t dt = tmem + buf * BN;
           const int kend = min(nkb, (cc + 1) * chunk);
-          for (int i = 0, kb = cc * chunk; kb < kend; ++i, ++kb, ++it) {
-            const int s = static_cast<int>(it % STAGES);
-            const uint32_t ph = static_cast<uint32_t>(it / STAGES) & 1u;
+          for (int i = 0, kb = cc * chunk; kb < kend; ++i, ++kb) {
             if (!mbar_wait(&full[s], ph, wait_ns)) {
               atomicExch(err, 1);
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t a0 = smem_u32(smem + s * STAGE_BYTES);
-            const uint32_t b0 = a0 + A_BYTES;
-            const uint32_t alo = b0 + B_BYTES;
-            const uint32_t blo = alo + A_BYTES;
+            // descriptor addresses count 16 bytes: hi A, hi B, lo A, lo B
+            const uint64_t da = desc0 + static_cast<uint32_t>(s * (STAGE_BYTES >> 4));
+            const uint64_t db = da + (A_BYTES >> 4);
+            const uint64_t dal = db + (B_BYTES >> 4), dbl = dal + (A_BYTES >> 4);
 #pragma unroll
             for (int kk = 0; kk < ROW_BYTES / MMA_K_BYTES; ++kk) {
-              const uint64_t da = sw128_desc(a0 + kk * MMA_K_BYTES);
-              const uint64_t db = sw128_desc(b0 + kk * MMA_K_BYTES);
-              mma<F16K, PAIR>(dt, da, db, IDESC, (i > 0 || kk > 0) ? 1u : 0u);
+              constexpr int KD = MMA_K_BYTES >> 4;
+              mma<F16K, PAIR>(dt, da + kk * KD, db + kk * KD, IDESC, (i > 0 || kk > 0) ? 1u : 0u);
               if constexpr (SPLIT) {
-                mma<F16K, PAIR>(dt, da, sw128_desc(blo + kk * MMA_K_BYTES), IDESC, 1u);
-                mma<F16K, PAIR>(dt, sw128_desc(alo + kk * MMA_K_BYTES), db, IDESC, 1u);
+                mma<F16K, PAIR>(dt, da + kk * KD, dbl + kk * KD, IDESC, 1u);
+                mma<F16K, PAIR>(dt, dal + kk * KD, db + kk * KD, IDESC, 1u);
               }
             }
             mma_commit_both<PAIR>(&empty[s]);
+            if (++s == STAGES) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
           mma_commit_both<PAIR>(&tfull[buf]);
         }
