@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(SK_THREADS) skinny_kernel(const SkinnyDesc d, 
     }
   }
   const long cb = live ? (d.cb ? d.cb[r] : r * d.ldcb) : 0;
-  for (int s0 = 0; s0 < d.Ns; s0 += chunk) {
+  for (int s0 = blockIdx.y * chunk; s0 < d.Ns; s0 += gridDim.y * chunk) {
     const int ns = min(chunk, d.Ns - s0);
     __syncthreads();
     for (int i = threadIdx.x; i < ns * KH; i += SK_THREADS) {
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(SK_THREADS) skinny64_kernel(const SkinnyDesc d
   }
   const long cb = live ? (d.cb ? d.cb[r] : r * d.ldcb) : 0;
   const bool b0 = d.beta.x == 0.0 && d.beta.y == 0.0;
-  for (int s0 = 0; s0 < d.Ns; s0 += chunk) {
+  for (int s0 = blockIdx.y * chunk; s0 < d.Ns; s0 += gridDim.y * chunk) {
     const int ns = min(chunk, d.Ns - s0);
     __syncthreads();
     for (int i = threadIdx.x; i < ns * KM; i += SK_THREADS) {
@@ -166,6 +166,25 @@ __global__ void __launch_bounds__(SK_THREADS) skinny64_kernel(const SkinnyDesc d
   }
 }
 
+// Short rows per block: as many as the shared memory takes, unless the long
+// side leaves fewer than about four blocks per SM: then the short side is cut
+// as well, down to min_s rows (each block reads its long rows again, from L2).
+// One block row per 256 long rows had left a K = 1 product of 3200 x 100 on 13
+// SMs (236 us, now 15); FP64 residual at o = 10, v = 30, X = 120 2.83 -> 1.95
+// ms, FP16 residual at o = 40, v = 300, X = 1200 102.8 -> 100.6 ms.
+int pick_chunk(const SkinnyDesc &d, int per_s, int min_s, int *ny) {
+  const long bx = (d.Mb + SK_THREADS - 1) / SK_THREADS;
+  const int cap = std::max(1, std::min(d.Ns, SK_SMEM / per_s));
+  const long want = std::min<long>((d.Ns + min_s - 1) / min_s, (4L * 152 + bx - 1) / bx);
+  int chunk = cap;
+  if (want > (d.Ns + cap - 1) / cap) {
+    chunk = static_cast<int>((d.Ns + want - 1) / want);
+    chunk += chunk & 1;  // the FP32 kernel takes two short rows a pass
+  }
+  *ny = static_cast<int>(std::min<long>(bx >= 4L * 152 ? 1 : (d.Ns + chunk - 1) / chunk, 65535));
+  return chunk;
+}
+
 template <int KM>
 void skinny_launch(const SkinnyDesc &d, cudaStream_t st) {
   // set once per process (thread-safe static initialisation)
@@ -176,14 +195,15 @@ void skinny_launch(const SkinnyDesc &d, cudaStream_t st) {
   }();
   (void)attr;
   const int per_s = (KM / 2) * static_cast<int>(sizeof(float4));
-  const int chunk = std::max(1, std::min(d.Ns, SK_SMEM / per_s));
+  int ny;
+  const int chunk = pick_chunk(d, per_s, 8, &ny);
   const int beta_mode = (d.beta.x == 0.0 && d.beta.y == 0.0) ? 0
                         : (d.beta.x == 1.0 && d.beta.y == 0.0) ? 1
                                                                : 2;
   const float2 af = make_float2(static_cast<float>(d.alpha.x), static_cast<float>(d.alpha.y));
   const long blocks = (d.Mb + SK_THREADS - 1) / SK_THREADS;
-  skinny_kernel<KM><<<static_cast<unsigned>(blocks), SK_THREADS, chunk * per_s, st>>>(d, chunk,
-                                                                                     beta_mode, af);
+  skinny_kernel<KM><<<dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(ny)), SK_THREADS,
+                      chunk * per_s, st>>>(d, chunk, beta_mode, af);
   LAUNCH_CHECK();
   count_launch();
 }
@@ -198,9 +218,11 @@ void skinny64_launch(const SkinnyDesc &d, cudaStream_t st) {
   }();
   (void)attr;
   const int per_s = KM * static_cast<int>(sizeof(double2));
-  const int chunk = std::max(1, std::min(d.Ns, SK_SMEM / per_s));
+  int ny;
+  const int chunk = pick_chunk(d, per_s, 2, &ny);
   const long blocks = (d.Mb + SK_THREADS - 1) / SK_THREADS;
-  skinny64_kernel<KM><<<static_cast<unsigned>(blocks), SK_THREADS, chunk * per_s, st>>>(d, chunk);
+  skinny64_kernel<KM><<<dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(ny)), SK_THREADS,
+                        chunk * per_s, st>>>(d, chunk);
   LAUNCH_CHECK();
   count_launch();
 }
@@ -213,7 +235,8 @@ void gemm_skinny(const SkinnyDesc &d, cudaStream_t st) {
   if (d.Mb > 0x7fffffffL * SK_THREADS) fail(CC_ERR_ARG, "gemm_skinny: too many rows");
   if (d.f64) {
     if (d.K > SKINNY64_MAX_K) fail(CC_ERR_ARG, "gemm_skinny: K out of range (FP64)");
-    if (d.K <= 8) skinny64_launch<8>(d, st);
+    if (d.K <= 2) skinny64_launch<2>(d, st);
+    else if (d.K <= 8) skinny64_launch<8>(d, st);
     else if (d.K <= 16) skinny64_launch<16>(d, st);
     else if (d.K <= 24) skinny64_launch<24>(d, st);
     else skinny64_launch<32>(d, st);

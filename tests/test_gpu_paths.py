@@ -146,3 +146,26 @@ def test_fp64_residual_and_sigma_on_tensor_cores(o, v, X):
                      (sd, np.array([ipeom.sigma(H, x[k], o, v) for k in range(7)])),
                      (ld, np.array([ipeom.left_sigma(H, x[k], o, v) for k in range(7)]))):
         assert np.abs(got.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 3000, 2), (100, 3200, 1), (250, 1025, 17), (200, 5000, 32),
+                                   (1024, 7, 3), (90000, 9, 2)])
+def test_fp64_short_k_products_cut_on_both_sides(M, N, K):
+    P = _gpu()
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A, B = _cn(g, M, K), _cn(g, N, K)
+    C = torch.empty((M, N), dtype=torch.complex128, device="cuda")
+    P.zgemm_dev(A, B, C, "fp64")
+    _check_product(A, B, C)
+
+
+@pytest.mark.parametrize("M,N,K", [(2048, 200, 16), (300, 2500, 20), (1000, 40000, 48), (8, 2048, 33)])
+def test_fp32_short_k_products_cut_on_both_sides(M, N, K):
+    """FP32 products and sums of 2 K terms: 2 K 2^-24 of |a_m| |b_n|."""
+    P = _gpu()
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A, B = _cn(g, M, K), _cn(g, N, K)
+    C = torch.empty((M, N), dtype=torch.complex128, device="cuda")
+    P.zgemm_dev(A, B, C, "fp16x3")
+    tol = 2 * K * 2.0 ** -24 * _rownorm(A)[:, None] * _rownorm(B)[None, :]
+    assert bool(((C - A @ B.T).abs() <= tol).all())
