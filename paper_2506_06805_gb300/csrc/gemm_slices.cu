@@ -476,9 +476,11 @@ struct SideArgs {
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
 // e[row] = the largest exponent field of the row's components (at least 1),
-// e[rows] != 0 if any is 2047. One warp per item: 32 rows x 64 k with lanes
-// along the rows where those are neighbours in memory, else one row x 1024 k
-// with lanes along k. HBM bound: one read of the operand.
+// e[rows] != 0 if any is 2047. One warp per item: 32 rows x 16 k with lanes
+// along the rows where those are neighbours in memory, else one row x 256 k
+// with lanes along k, 8 loads in flight: on small operands the time is one
+// item's latency (items four times as long took 36 us at any size), on
+// large ones the read of the operand.
 __global__ void __launch_bounds__(256) slice_exp_kernel(SideArgs a, SideArgs b, long K, long items_a,
                                                         long items) {
   const int lane = threadIdx.x & 31;
@@ -488,11 +490,11 @@ __global__ void __launch_bounds__(256) slice_exp_kernel(SideArgs a, SideArgs b, 
     const long it = w < items_a ? w : w - items_a;
     int m = 1;
     if (s.rows_unit) {
-      const long nk = (K + 63) / 64;
-      const long r = (it / nk) * 32 + lane, k0 = (it % nk) * 64, k1 = min(K, k0 + 64);
+      const long nk = (K + 15) / 16;
+      const long r = (it / nk) * 32 + lane, k0 = (it % nk) * 16, k1 = min(K, k0 + 16);
       if (r < s.rows) {
         const long ro = s.rt ? s.rt[r] : r * s.ld;
-#pragma unroll 4
+#pragma unroll 8
         for (long k = k0; k < k1; ++k) {
           const double2 x = s.src[ro + (s.kt ? s.kt[k] : k)];
           m = max(m, max(exp_field(x.x), exp_field(x.y)));
@@ -501,10 +503,10 @@ __global__ void __launch_bounds__(256) slice_exp_kernel(SideArgs a, SideArgs b, 
         if (m == 2047) s.e[s.rows] = 1;
       }
     } else {
-      const long nk = (K + 1023) / 1024;
-      const long r = it / nk, k0 = (it % nk) * 1024, k1 = min(K, k0 + 1024);
+      const long nk = (K + 255) / 256;
+      const long r = it / nk, k0 = (it % nk) * 256, k1 = min(K, k0 + 256);
       const long ro = s.rt ? s.rt[r] : r * s.ld;
-#pragma unroll 4
+#pragma unroll 8
       for (long k = k0 + lane; k < k1; k += 32) {
         const double2 x = s.src[ro + (s.kt ? s.kt[k] : k)];
         m = max(m, max(exp_field(x.x), exp_field(x.y)));
@@ -717,7 +719,7 @@ void slice_pack(const SliceOperand *A, const SlicePlanes *pa, const SliceOperand
   auto setup = [&](const SliceOperand &x, const SlicePlanes &p, bool expand, SideArgs &s, long &ne,
                    long &nt) {
     s = side(x, p, expand);
-    ne = x.rows_unit ? (x.rows + 31) / 32 * ((K + 63) / 64) : x.rows * ((K + 1023) / 1024);
+    ne = x.rows_unit ? (x.rows + 31) / 32 * ((K + 15) / 16) : x.rows * ((K + 255) / 256);
     nt = (x.rows + 31) / 32 * (p.Kp / 64);
     Kp = p.Kp;
     CUDA_CHECK(cudaMemsetAsync(p.e, 0, sizeof(int) * (2 * x.rows + 1), st));
@@ -825,19 +827,23 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
 }
 
 // Estimated times (s) of an M x N x K product here and on the FP64 pipe. The
-// tensor side: 28 digit products of every 256 x 128 x 64 block at about 1.3
+// tensor side: 28 digit products of every 128 x 128 x 64 block at about 1
 // PF/s, an epilogue of three K blocks per tile, the planes written and read,
-// five launches. The FP64 side: 1 TF/s or its operands at 5 TB/s, which is
-// its best case, so a product near the line does not lose by the change.
+// five launches. The FP64 side: 1 TF/s or its operands at 5 TB/s, on whole
+// 64 x 64 tiles where the tiled kernel takes the product (a tile's rows cost
+// the same empty: 5 x 64000 x 160 took 4.5 ms there).
 bool slices_pay(long M, long N, long K) {
   const double m = (2 * M + 127) / 128 * 128.0, n = (N + 127) / 128 * 128.0;
   const double kb = static_cast<double>((2 * K + 63) / 64);
-  const double mma = 2.0 * m * n * 64.0 * 28.0 * (kb + 3.0) / 1.3e15;
+  const double mma = 2.0 * m * n * 64.0 * 28.0 * (kb + 3.0) / 1e15;
   const double pack = (static_cast<double>(M) * K * (32 + 112) + static_cast<double>(N) * K * (32 + 56)) / 5e12;
   const double out = 32.0 * M * N / 5e12;
-  const double t_slices = 15e-6 + std::max(mma, 28.0 * 2.5e-7) + pack + out;
-  const double t_f64 = 4e-6 + std::max(8.0 * M * N * static_cast<double>(K) / 1e12,
-                                       16.0 * (static_cast<double>(M) * K + static_cast<double>(N) * K) / 5e12);
+  const double t_slices = 20e-6 + std::max(mma, 20e-6) + pack + out;
+  const long tm = (M + 63) / 64, tn = (N + 63) / 64;
+  const bool skinny = K <= SKINNY64_MAX_K && std::min(M, N) <= 256 && std::max(M, N) >= 1024;
+  const bool tiled = M > 1 && N > 1 && !skinny && tm * tn >= 152;
+  const double mn = tiled ? 4096.0 * tm * tn : static_cast<double>(M) * N;
+  const double t_f64 = 4e-6 + std::max(8.0 * mn * K / 1e12, 16.0 * (static_cast<double>(M) * K + static_cast<double>(N) * K) / 5e12);
   return t_slices < 0.8 * t_f64;
 }
 
