@@ -12,19 +12,20 @@
 // two rows' largest magnitudes per term. Each digit product is at most 2^16
 // in magnitude, so 256 of them (four K blocks of 64) add up without any
 // rounding in the FP32 accumulators of tcgen05.mma; the epilogue warps then
-// move the sums out of TMEM: groups 7 .. EX + 1 into FP32 (their rounding
-// lies 2^-24 below 2^(-9 EX) of the result), groups EX .. 1 into 64-bit
-// integers, exactly. EX is 5 where the rows' and columns' 2-norms bound the
-// integers below 2^63 (Cauchy-Schwarz; the norms, relative to 2^E, come from
-// the packing), else 4; the sum may wrap on the way, only its value counts.
+// move the sums out of TMEM: groups 7 and 6 into FP32 (whose rounding lies
+// 2^-24 below 2^-45 of the result), groups 5 .. 1 into 64-bit integers. Those
+// are exact while the rows' and columns' 2-norms (relative to 2^E, from the
+// packing) bound the sum below 2^62; for the larger ones of long, even rows,
+// group 5 joins the FP32 part. The sum may wrap on the way, only its value
+// counts.
 //
 // Accuracy, RMS error over |a_m| |b_n| against quadruple precision, here and
 // from the FP64 kernel, normal operands: K = 160 7.9e-18 / 1.3e-17, K = 1200
 // 2.7e-18 / 6.0e-18, K = 20000 1.1e-18 / 4.3e-18.
 //
 // Measured against the FP64 kernels: product of 1536 x 1000 x 1200 14.7 ->
-// 1.3 ms, ladder at o = 15, v = 131, X = 517 983 -> 38 ms, FP64 residual at
-// o = 12, v = 72, X = 288 80.7 -> 9.0 ms.
+// 0.88 ms, ladder at o = 15, v = 131, X = 517 983 -> 22 ms, FP64 residual at
+// o = 12, v = 72, X = 288 80.7 -> 5.3 ms.
 //
 // Rows that hold an Inf or NaN cannot be cut: the packing raises a flag on
 // the device, the slice kernel then stores nothing, and a guarded launch of
@@ -43,15 +44,18 @@ namespace {
 
 constexpr int NS = SLICE_COUNT;  // digits per element
 constexpr int SBN = 128;         // output columns per tile
-constexpr int CHUNK = 4;         // K blocks per TMEM accumulation (256 terms)
+constexpr int SKB = 2;           // K blocks of 64 per shared-memory slot and step
+constexpr int CHUNK = 2;         // steps per TMEM accumulation (at most 256 terms)
 constexpr int NBUF = 3;          // TMEM accumulators in flight (128 columns each)
+constexpr int BAR_BYTES = 512;  // barriers
 constexpr uint32_t STASH = NBUF * SBN;  // TMEM columns that hold the FP32 part
 
-// 12 warps: 0-7 epilogue, 8 TMA producer, 9 MMA issuer, 10-11 idle (they
-// complete the warpgroup that gives registers away). Launched with 168
-// registers a thread (64512 in all); warps 8-11 drop to 56, the epilogue's
-// 256 threads rise to 224: 256 x 224 + 128 x 56 = 64512.
-constexpr int SLICE_THREADS = 384;
+// 20 warps: 0-15 epilogue, 16 TMA producer of A, 17 MMA issuer, 18 TMA
+// producer of B, 19 idle (it completes the warpgroup that gives registers
+// away). Launched with 96 registers a thread (61440 in all); warps 16-19 drop
+// to 48, the epilogue's 512 threads rise to 104: 512 x 104 + 128 x 48 = 59392.
+constexpr int EPI_WARPS = 16;
+constexpr int SLICE_THREADS = (EPI_WARPS + 4) * 32;
 
 enum { SW_STORE = 0, SW_ADD = 1, SW_BETA = 2 };
 
@@ -88,6 +92,17 @@ __device__ __forceinline__ void slice_coords(const SliceArgs &a, int t, int &m, 
   n = r / gsize;
 }
 
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
+  uint32_t r[4];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float *v) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
@@ -101,6 +116,8 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float *v) {
       : "memory");
 }
 
+__device__ __noinline__ double scale_slow(double d, int e) { return scalbn(d, e); }
+
 // d 2^e; the exponent field is adjusted in place unless the value or the
 // result is not a normal number
 __device__ __forceinline__ double scale_exp(double d, int e) {
@@ -109,7 +126,7 @@ __device__ __forceinline__ double scale_exp(double d, int e) {
   const int ne = ex + e;
   if (ex != 0 && ne > 0 && ne < 2047)
     return __hiloint2double(hi + (e << 20), __double2loint(d));
-  return scalbn(d, e);
+  return scale_slow(d, e);
 }
 
 // t as a double, rounded to nearest even, on the integer pipes (the hardware
@@ -128,34 +145,59 @@ __device__ __forceinline__ double i64_to_f64(long long t) {
   return __longlong_as_double(static_cast<long long>(b | s));
 }
 
-// Persistent CTA or CTA pair, warps as in tc_gemm_kernel (gemm_tc.cu): 0-7
-// epilogue, 8 TMA producer, 9 TMEM allocator and MMA issuer; every wait
-// bounded. Tiles of UNIT_ROWS real rows x 128 columns: 64-bit sums for 256
-// columns would not fit the epilogue's registers. A pair's MMA (256 x 128)
-// then reads 96 B of shared memory per SM clock and the copies write as
-// much, the same as tc_gemm_kernel's 128 x 256 single-CTA tile. Per tile the
-// groups run from 7 to 1, and in each the digit pairs (i, g + 1 - i) over
-// the K range, cut into TMEM chunks of four K blocks regardless of the pair.
+// The order of the digit products, shared by the three roles. Groups go in
+// pairs (G, G - 1) for G = 7, 5, 3, 1, and within a K block the 2 G - 1
+// products of such a pair zigzag through the digits,
+//   (A_1, B_G), (A_1, B_G-1), (A_2, B_G-1), (A_2, B_G-2), ..., (A_G, B_1):
+// even steps belong to group G, odd ones to G - 1, and each step brings in
+// one new digit plane block, A on even steps, B on odd ones. A group's
+// products collect in a TMEM buffer of its own, CHUNK of them at a time. A
+// "K block" of this order is SKB blocks of 64 (one at the end of an odd
+// range).
+struct BufQueue {  // free TMEM buffers in the order they were handed over
+  uint32_t q = 0u | (1u << 2) | (2u << 4);
+  int n = NBUF;
+  __device__ __forceinline__ int pop() {
+    const int b = q & 3u;
+    q >>= 2;
+    --n;
+    return b;
+  }
+  __device__ __forceinline__ void push(int b) { q |= static_cast<uint32_t>(b) << (2 * n++); }
+};
+
+// Persistent CTA or CTA pair, roles as in tc_gemm_kernel (gemm_tc.cu); every
+// wait bounded. Tiles of UNIT_ROWS real rows x 128 columns: 64-bit sums for
+// 256 columns would not fit the epilogue's registers. Such a tile needs 24 KB
+// of operands per 256 clocks of MMA, about twice what L2 delivers; the
+// zigzag uses every block of a plane twice and halves that. A step costs its
+// single issuing threads a few hundred clocks of instructions and barrier
+// round trips, so it spans two K blocks, 512 clocks of MMA. The epilogue
+// (an integer conversion and a 64-bit add for every value of every chunk)
+// needs four warps a scheduler to keep up. Kernel alone, 4096 x 4096 x K
+// (group by group with eight epilogue warps -> this): K = 512 2.41 -> 1.58
+// ms, K = 2048 6.46 -> 5.46 ms, 400 clocks a K block where the MMAs take 256.
 template <int STAGES, bool PAIR>
 __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __grid_constant__ SliceArgs P) {
-  constexpr int A_BYTES = BM * ROW_BYTES;
-  constexpr int B_BYTES = (PAIR ? SBN / 2 : SBN) * ROW_BYTES;
-  constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  constexpr int A_BLK = BM * ROW_BYTES;  // one K block
+  constexpr int B_BLK = (PAIR ? SBN / 2 : SBN) * ROW_BYTES;
+  constexpr int A_BYTES = SKB * A_BLK, B_BYTES = SKB * B_BLK;  // one slot
   constexpr int UNIT_ROWS = PAIR ? 2 * BM : BM;
   constexpr uint32_t IDESC = make_idesc(UNIT_ROWS, SBN, 0u);
-  constexpr int HALF = SBN / 2;  // columns per epilogue warp
+  constexpr int COLS = SBN * 4 / EPI_WARPS;  // columns per epilogue warp
   constexpr uint32_t TMEM_COLS = 512;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES);
-  uint64_t *empty = full + STAGES;
-  uint64_t *tfull = empty + STAGES;    // [NBUF]
+  uint8_t *smem_b = smem + STAGES * A_BYTES;  // rings of A and of B blocks
+  uint64_t *fullA = reinterpret_cast<uint64_t *>(smem + STAGES * (A_BYTES + B_BYTES));
+  uint64_t *fullB = fullA + STAGES, *emptyA = fullB + STAGES, *emptyB = emptyA + STAGES;
+  uint64_t *tfull = emptyB + STAGES;   // [NBUF]
   uint64_t *tempty = tfull + NBUF;     // [NBUF]
   uint64_t *mdone = tempty + NBUF;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mdone + 1);
-  double *stage = reinterpret_cast<double *>(smem + STAGES * STAGE_BYTES + 256);  // 8 x 4 KB
+  long long *stage = reinterpret_cast<long long *>(smem + STAGES * (A_BYTES + B_BYTES) + BAR_BYTES);  // 1.5 KB a warp
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -166,153 +208,192 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+      mbar_init(&fullA[s], 1);
+      mbar_init(&fullB[s], 1);
+      mbar_init(&emptyA[s], 1);
+      mbar_init(&emptyB[s], 1);
     }
     for (int b = 0; b < NBUF; ++b) {
       mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], PAIR ? 16 : 8);
+      mbar_init(&tempty[b], PAIR ? 2 * EPI_WARPS : EPI_WARPS);
     }
     mbar_init(mdone, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp == 9) tmem_alloc<PAIR>(tmem_slot, TMEM_COLS);
+  if (warp == EPI_WARPS + 1) tmem_alloc<PAIR>(tmem_slot, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   if constexpr (PAIR) cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-    if (warp == 8) {
+  if (warp >= EPI_WARPS) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    if (warp == EPI_WARPS || warp == EPI_WARPS + 2) {
       if (lane == 0) {
-        // ---------------- TMA producer ----------------
-        long it = 0;
+        // ---------------- TMA producers of A and of B ----------------
+        const bool is_a = warp == EPI_WARPS;
+        uint64_t *const full = is_a ? fullA : fullB, *const empty = is_a ? emptyA : emptyB;
+        uint8_t *const ring = is_a ? smem : smem_b;
+        const CUtensorMap *const map = is_a ? &P.mA : &P.mB;
+        const int blk = is_a ? A_BLK : B_BLK;
+        const int rows = static_cast<int>(is_a ? P.rows_a : P.rows_b);
+        long n = 0;  // slots filled
         int s = 0;
-        uint32_t ph = 1;  // parity of the wait for a free stage
+        uint32_t par = 1;  // parity of the wait for a free slot
         bool ok = true;
         for (int t = TC_UNIT0; t < n_units && ok; t += TC_USTEP) {
           int m_tile, n_tile, z;
           slice_coords(P, t, m_tile, n_tile, z);
           const int kb0 = z * P.kb_per_split;
           const int kb1 = min(P.num_kb, kb0 + P.kb_per_split);
-          const int ya = static_cast<int>(P.a_row0) + m_tile * UNIT_ROWS + TC_RANK * BM;
-          const int yb = static_cast<int>(P.b_row0) + n_tile * SBN + (PAIR ? TC_RANK * (SBN / 2) : 0);
-          for (int g = NS; g >= 1 && ok; --g)
-            for (int p = 0; p < g && ok; ++p) {
-              const int yap = ya + p * static_cast<int>(P.rows_a);
-              const int ybp = yb + (g - 1 - p) * static_cast<int>(P.rows_b);
-              for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                if (!mbar_wait(&empty[s], ph, P.wait_ns)) {
+          const int y = is_a ? static_cast<int>(P.a_row0) + m_tile * UNIT_ROWS + TC_RANK * BM
+                             : static_cast<int>(P.b_row0) + n_tile * SBN + (PAIR ? TC_RANK * (SBN / 2) : 0);
+          for (int G = NS; G >= 1 && ok; G -= 2)
+            for (int kb = kb0; kb < kb1 && ok; kb += SKB) {
+              const int nb = min(SKB, kb1 - kb);
+              int yi = is_a ? y : y + (G - 1) * rows;  // A's digits ascend, B's descend
+              for (int i = 0; i < G; ++i, yi += is_a ? rows : -rows) {
+                if (!mbar_wait(&empty[s], par, P.wait_ns)) {
                   atomicExch(P.err, 1);
                   ok = false;
                   break;
                 }
-                uint8_t *st = smem + s * STAGE_BYTES;
+                uint8_t *dst = ring + s * SKB * blk;
                 if constexpr (PAIR) {
-                  if (TC_RANK == 0) mbar_expect_tx(&full[s], 2 * STAGE_BYTES);
+                  if (TC_RANK == 0) mbar_expect_tx(&full[s], 2 * nb * blk);
                   const uint32_t fb = leader_addr(smem_u32(&full[s]));
-                  tma_load_2d_pair(st, &P.mA, fb, kb * 64, yap);
-                  tma_load_2d_pair(st + A_BYTES, &P.mB, fb, kb * 64, ybp);
+                  tma_load_2d_pair(dst, map, fb, kb * 64, yi);
+                  if (nb == 2) tma_load_2d_pair(dst + blk, map, fb, kb * 64 + 64, yi);
                 } else {
-                  mbar_expect_tx(&full[s], STAGE_BYTES);
-                  tma_load_2d(st, &P.mA, &full[s], kb * 64, yap);
-                  tma_load_2d(st + A_BYTES, &P.mB, &full[s], kb * 64, ybp);
+                  mbar_expect_tx(&full[s], nb * blk);
+                  tma_load_2d(dst, map, &full[s], kb * 64, yi);
+                  if (nb == 2) tma_load_2d(dst + blk, map, &full[s], kb * 64 + 64, yi);
                 }
+                ++n;
                 if (++s == STAGES) {
                   s = 0;
-                  ph ^= 1u;
+                  par ^= 1u;
                 }
               }
             }
         }
         // no copy may outlive the CTA's shared memory (see tc_gemm_kernel)
-        if (TC_RANK == 0) {
-          for (long i = (it > STAGES ? it - STAGES : 0); i < it; ++i) {
+        if (TC_RANK == 0)
+          for (long i = (n > STAGES ? n - STAGES : 0); i < n; ++i)
             if (!mbar_wait(&full[i % STAGES], static_cast<uint32_t>(i / STAGES) & 1u, DRAIN_NS))
               atomicExch(P.err, 1);
-          }
-        }
       }
-    } else if (warp == 9) {
+    } else if (warp == EPI_WARPS + 1) {
       if (TC_RANK == 0 && elect_one()) {
         // ---------------- MMA issuer (the leader of a pair) ----------------
-        long c = 0;
-        int buf = 0, s = 0;
-        uint32_t bph = 0, ph = 0;  // parities of the TMEM buffers and the stages
+        BufQueue bq;
+        uint32_t waits = 0, par = 0;  // per TMEM buffer: used before; parity of its next release
+        int sa = STAGES - 1, sb = STAGES - 1;  // slots in use
+        uint32_t pa = 1, pb = 1;               // parities of their fills
         bool ok = true;
-        const uint64_t desc0 = sw128_desc(smem_u32(smem));
+        const uint64_t desc_a = sw128_desc(smem_u32(smem)), desc_b = sw128_desc(smem_u32(smem_b));
+        auto next_a = [&] {
+          if (++sa == STAGES) {
+            sa = 0;
+            pa ^= 1u;
+          }
+          return mbar_wait(&fullA[sa], pa, P.wait_ns);
+        };
+        auto next_b = [&] {
+          if (++sb == STAGES) {
+            sb = 0;
+            pb ^= 1u;
+          }
+          return mbar_wait(&fullB[sb], pb, P.wait_ns);
+        };
+        // the product of the two current slots, collected in its group's buffer
+        auto product = [&](int nb, int &cnt, int &buf) {
+          if (cnt == 0) {
+            buf = bq.pop();
+            if ((waits >> buf) & 1u) {
+              if (!mbar_wait(&tempty[buf], (par >> buf) & 1u, P.wait_ns)) return false;
+              par ^= 1u << buf;
+            }
+            waits |= 1u << buf;
+          }
+          tc_fence_after();
+          const uint64_t da = desc_a + static_cast<uint32_t>(sa * (A_BYTES >> 4));  // in 16 bytes
+          const uint64_t db = desc_b + static_cast<uint32_t>(sb * (B_BYTES >> 4));
+          const uint32_t dt = tmem + buf * SBN;
+#pragma unroll
+          for (int kk = 0; kk < ROW_BYTES / 32; ++kk)
+            mma<true, PAIR>(dt, da + 2 * kk, db + 2 * kk, IDESC, (cnt > 0 || kk > 0) ? 1u : 0u);
+          if (nb == 2) {
+#pragma unroll
+            for (int kk = 0; kk < ROW_BYTES / 32; ++kk)
+              mma<true, PAIR>(dt, da + (A_BLK >> 4) + 2 * kk, db + (B_BLK >> 4) + 2 * kk, IDESC, 1u);
+          }
+          ++cnt;
+          return true;
+        };
+        auto hand_over = [&](int &cnt, int buf) {
+          mma_commit_both<PAIR>(&tfull[buf]);
+          bq.push(buf);
+          cnt = 0;
+        };
         for (int t = TC_UNIT0; t < n_units && ok; t += TC_USTEP) {
           int m_tile, n_tile, z;
           slice_coords(P, t, m_tile, n_tile, z);
           const int kb0 = z * P.kb_per_split;
           const int nkb = min(P.num_kb, kb0 + P.kb_per_split) - kb0;
-          for (int g = NS; g >= 1 && ok; --g) {
-            for (int left = g * nkb; left > 0 && ok; left -= CHUNK, ++c) {
-              if (c >= NBUF && !mbar_wait(&tempty[buf], bph ^ 1u, P.wait_ns)) {
-                atomicExch(P.err, 1);
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-              const uint32_t dt = tmem + buf * SBN;
-              const int nb = min(left, CHUNK);
-              for (int i = 0; i < nb; ++i) {
-                if (!mbar_wait(&full[s], ph, P.wait_ns)) {
-                  atomicExch(P.err, 1);
-                  ok = false;
+          for (int G = NS; G >= 1 && ok; G -= 2) {
+            int cnt0 = 0, cnt1 = 0, buf0 = 0, buf1 = 0;  // groups G and G - 1
+            for (int kb = 0; kb < nkb && ok; kb += SKB) {
+              const int nb = min(SKB, nkb - kb);
+              ok = next_a() && next_b();
+              for (int i = 0; ok; ++i) {
+                if (!(ok = product(nb, cnt0, buf0))) break;
+                mma_commit_both<PAIR>(&emptyB[sb]);
+                if (cnt0 == CHUNK) hand_over(cnt0, buf0);
+                if (i == G - 1) {
+                  mma_commit_both<PAIR>(&emptyA[sa]);
                   break;
                 }
-                tc_fence_after();
-                // descriptor addresses count 16 bytes
-                const uint64_t da = desc0 + static_cast<uint32_t>(s * (STAGE_BYTES >> 4));
-#pragma unroll
-                for (int kk = 0; kk < ROW_BYTES / 32; ++kk)
-                  mma<true, PAIR>(dt, da + 2 * kk, da + (A_BYTES >> 4) + 2 * kk, IDESC,
-                                  (i > 0 || kk > 0) ? 1u : 0u);
-                mma_commit_both<PAIR>(&empty[s]);
-                if (++s == STAGES) {
-                  s = 0;
-                  ph ^= 1u;
-                }
-              }
-              mma_commit_both<PAIR>(&tfull[buf]);
-              if (++buf == NBUF) {
-                buf = 0;
-                bph ^= 1u;
+                if (!(ok = next_b() && product(nb, cnt1, buf1))) break;
+                mma_commit_both<PAIR>(&emptyA[sa]);
+                if (cnt1 == CHUNK) hand_over(cnt1, buf1);
+                ok = next_a();
               }
             }
+            if (ok && cnt0) hand_over(cnt0, buf0);
+            if (ok && cnt1) hand_over(cnt1, buf1);
           }
         }
+        if (!ok) atomicExch(P.err, 1);
         mma_commit_self<PAIR>(mdone);
         if (!mbar_wait(mdone, 0u, DRAIN_NS)) atomicExch(P.err, 1);
       }
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
-    // ---------------- epilogue: 8 warps ----------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+    // ---------------- epilogue ----------------
     const int q = warp & 3;
     const int h = warp >> 2;
     const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
-    int buf = 0;
-    uint32_t bph = 0;
+    BufQueue bq;
+    uint32_t par = 0;  // per TMEM buffer: parity of its next filling
     bool ok = true;
-    // one chunk: wait for it, hand its 64 columns to f(column, value), free it
-    auto drain = [&](auto &&f) {
-      if (!mbar_wait(&tfull[buf], bph, P.wait_ns)) {
+    // one chunk: wait for it, hand 16 columns at a time to f(column, values), free it
+    auto drain = [&](int buf, auto &&f) {
+      if (!mbar_wait(&tfull[buf], (par >> buf) & 1u, P.wait_ns)) {
         ok = false;
         return;
       }
+      par ^= 1u << buf;
       tc_fence_after();
-      const uint32_t base = tmem + lanes + buf * SBN + h * HALF;
+      const uint32_t base = tmem + lanes + buf * SBN + h * COLS;
 #pragma unroll
-      for (int j = 0; j < HALF; j += 16) {
+      for (int j = 0; j < COLS; j += 16) {
         float v[16];
         tmem_ld16(base + j, v);
-#pragma unroll
-        for (int u = 0; u < 16; ++u) f(j + u, v[u]);
+        f(j, v);
       }
       tc_fence_before();
       __syncwarp();
@@ -322,9 +403,45 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
         else
           mbar_arrive(&tempty[buf]);
       }
-      if (++buf == NBUF) {
-        buf = 0;
-        bph ^= 1u;
+    };
+    // the chunks of groups (G, G - 1) in the issuer's order, each given to f
+    // (one place: the epilogue's unrolled code has to stay in the
+    // instruction cache)
+    auto chunks = [&](int G, int nkb, auto &&f) {
+      int cnt0 = 0, cnt1 = 0, buf0 = 0, buf1 = 0, p = 0, left = (nkb + SKB - 1) / SKB * (2 * G - 1);
+      while (ok) {
+        int buf = -1, g = G;
+        for (; left > 0 && buf < 0; --left) {
+          if ((p & 1) == 0) {
+            if (cnt0 == 0) buf0 = bq.pop();
+            if (++cnt0 == CHUNK) {
+              buf = buf0;
+              cnt0 = 0;
+            }
+          } else {
+            if (cnt1 == 0) buf1 = bq.pop();
+            if (++cnt1 == CHUNK) {
+              buf = buf1;
+              g = G - 1;
+              cnt1 = 0;
+            }
+          }
+          if (++p == 2 * G - 1) p = 0;
+        }
+        if (buf < 0) {  // the incomplete chunks at the end
+          if (cnt0) {
+            buf = buf0;
+            cnt0 = 0;
+          } else if (cnt1) {
+            buf = buf1;
+            g = G - 1;
+            cnt1 = 0;
+          } else {
+            break;
+          }
+        }
+        f(buf, g);
+        bq.push(buf);
       }
     };
     for (int t = TC_UNIT0; t < n_units && ok; t += TC_USTEP) {
@@ -335,103 +452,145 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
       // exponents (stored biased by 1022: row below 2^(e - 1022)) and norms
       // of this warp's rows and columns; those beyond the product are
       // computed on whatever the planes hold there and not stored
-      const long nbase = static_cast<long>(n_tile) * SBN + h * HALF;
+      const long nbase = static_cast<long>(n_tile) * SBN + h * COLS;
       const long mbase = (static_cast<long>(m_tile) * UNIT_ROWS + TC_RANK * BM) / 2 + q * 16;
       const long mrow = mbase + (lane >> 1);
-      bool ex5;
+      // the integers count 2^u last places of group 5, with |a| |b| 2^(52 - u)
+      // below 2^62 (u = 5 would make group 1's factor 2^31)
+      int u;
       {
         const float na = mrow < P.M ? P.na[P.a_row0 / 2 + mrow] : 0.f;
-        const float nb0 = nbase + lane < P.N ? P.nb[P.b_row0 + nbase + lane] : 0.f;
-        const float nb1 = nbase + 32 + lane < P.N ? P.nb[P.b_row0 + nbase + 32 + lane] : 0.f;
+        const float nb = nbase + lane < P.N ? P.nb[P.b_row0 + nbase + lane] : 0.f;
         const float a = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(na)));
-        const float b = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(nb0, nb1))));
-        ex5 = a * b < 0x1p19f;  // |a| |b| < 725: sums below 2^52 725 < 2^62
+        const float b = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(nb)));
+        const int e = static_cast<int>(__float_as_uint(a * b) >> 23) - 126;  // a b < 2^e
+        u = max(0, (e - 18) / 2);
+        if (u == 5) u = 6;
       }
       {
-        float lf[HALF];
+        float lf[COLS];
 #pragma unroll
-        for (int j = 0; j < HALF; ++j) lf[j] = 0.f;
-        for (int g = NS; g > (ex5 ? 5 : 4) && ok; --g) {
+        for (int j = 0; j < COLS; ++j) lf[j] = 0.f;
+        chunks(NS, nkb, [&](int buf, int g) {
+          const float w = g == NS ? 0x1p-9f : 1.0f;
+          drain(buf, [&](int j, const float (&x)[16]) {
 #pragma unroll
-          for (int j = 0; j < HALF; ++j) lf[j] *= 0x1p-9f;
-          for (int left = g * nkb; left > 0 && ok; left -= CHUNK)
-            drain([&](int j, float x) { lf[j] += x; });
-        }
+            for (int k = 0; k < 16; ++k) lf[j + k] = fmaf(w, x[k], lf[j + k]);
+          });
+        });
         if (!ok) break;
 #pragma unroll
-        for (int j = 0; j < HALF; j += 16) tmem_st16(tmem + lanes + STASH + h * HALF + j, lf + j);
+        for (int j = 0; j < COLS; j += 16) tmem_st16(tmem + lanes + STASH + h * COLS + j, lf + j);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       }
-      long long acc[HALF];
+      long long acc[COLS], bias = 0;
 #pragma unroll
-      for (int j = 0; j < HALF; ++j) acc[j] = 0;
-      // group g counts 2^(9 (EX - g)) in units of group EX's last place:
-      // group 1 in the upper word (36 places) or by a 32 x 32 -> 64 product
-      for (int g = ex5 ? 5 : 4; g >= 1 && ok; --g) {
-        const int sh = 9 * ((ex5 ? 5 : 4) - g);
-        if (sh < 32) {
-          const int mul = 1 << sh;
-          for (int left = g * nkb; left > 0 && ok; left -= CHUNK)
-            drain([&](int j, float x) {
-              asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc[j]) : "r"(__float2int_rn(x)), "r"(mul));
-            });
-        } else {
-          for (int left = g * nkb; left > 0 && ok; left -= CHUNK)
-            drain([&](int j, float x) {
-              const unsigned xi = static_cast<unsigned>(__float2int_rn(x)) << 4;
-              acc[j] += static_cast<long long>(static_cast<unsigned long long>(xi) << 32);
-            });
-        }
-      }
+      for (int j = 0; j < COLS; ++j) acc[j] = 0;
+      // A sum x below 2^22 becomes the integer MAGIC + x in the bits of
+      // x + 1.5 2^23 (the hardware conversion gives 16 values per clock and
+      // SM, a quarter of what the chunks need); larger ones, which a few
+      // hundred random digits do not reach, are converted. MAGIC times the
+      // factor is taken off once per tile.
+      constexpr int MAGIC = 0x4b400000;
+      for (int G = NS - 2; G >= 1; G -= 2)
+        chunks(G, nkb, [&](int buf, int g) {
+          const int sh = 9 * (5 - g) - u;
+          const int mul = 1 << min(max(sh, 0), 30);
+          const int up = sh - 32;
+          const bool fp = sh < 0;  // group 5 of a long, even row: to the FP32 part
+          if (!fp) bias += static_cast<long long>(static_cast<unsigned long long>(MAGIC) << max(sh, 0));
+          drain(buf, [&](int j, const float (&x)[16]) {
+            if (fp) {
+              float lf[16];
+              const uint32_t at = tmem + lanes + STASH + h * COLS + j;
+              tmem_ld16(at, lf);
+#pragma unroll
+              for (int k = 0; k < 16; ++k) lf[k] = fmaf(512.0f, x[k], lf[k]);
+              tmem_st16(at, lf);
+              asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+              return;
+            }
+            float m = 0.f;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) m = fmaxf(m, fabsf(x[k]));
+            int xi[16];
+            if (!__any_sync(0xffffffffu, m >= 0x1p22f)) {
+#pragma unroll
+              for (int k = 0; k < 16; ++k) xi[k] = __float_as_int(x[k] + 12582912.0f);
+            } else {
+#pragma unroll
+              for (int k = 0; k < 16; ++k) xi[k] = MAGIC + __float2int_rn(x[k]);
+            }
+            if (up < 0) {
+#pragma unroll
+              for (int k = 0; k < 16; ++k)
+                asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc[j + k]) : "r"(xi[k]), "r"(mul));
+            } else {
+#pragma unroll
+              for (int k = 0; k < 16; ++k)
+                acc[j + k] += static_cast<long long>(static_cast<unsigned long long>(static_cast<unsigned>(xi[k]) << up) << 32);
+            }
+          });
+        });
       if (!ok) break;
-      // value = (acc + 2^-9 lf) 2^(Ea + Eb - 16 - 9 (EX - 1))
+      // value = (2^(9 + u) acc + lf) 2^(Ea + Eb - 16 - 45), four columns at a
+      // time through shared memory: lane = real row on the way in, (row of
+      // eight, column) of complex results on the way out. The conversion
+      // sits on the way out, in a loop: unrolled over the accumulators it was
+      // far larger than the instruction cache (110 000 clocks a tile).
       const bool skip = (*P.fa | *P.fb) != 0;
-      const int ea = (mrow < P.M ? P.ea[P.a_row0 / 2 + mrow] : 1) - 2 * 1022 - 25 - (ex5 ? 36 : 27) +
-                     (P.alpha_p2 ? P.alpha_e : 0);
+      const int ea = (mrow < P.M ? P.ea[P.a_row0 / 2 + mrow] : 1) - 2 * 1022 - 61 + (P.alpha_p2 ? P.alpha_e : 0);
       const int ebl = nbase + lane < P.N ? P.eb[P.b_row0 + nbase + lane] : 1;
-      const int ebh = nbase + 32 + lane < P.N ? P.eb[P.b_row0 + nbase + 32 + lane] : 1;
       long roff = 0;
       if (lane < 16 && mbase + lane < P.M)
         roff = P.cm ? P.cm[mbase + lane] : (mbase + lane) * P.ldc;
-      double *stg = stage + warp * 512;  // 32 rows x 16 columns
-      const int col = lane & 15, hf = lane >> 4;
+      long long *sacc = stage + warp * 192;  // [32][4] integers, then [32][4] floats
+      float *slf = reinterpret_cast<float *>(sacc + 128);
+      const int col = lane & 3, hf = lane >> 2;
+#pragma unroll 1
+      for (int seg = 0; seg < COLS / 4; ++seg) {
+        float lf[4];
+        tmem_ld4(tmem + lanes + STASH + h * COLS + 4 * seg, lf);
 #pragma unroll
-      for (int j = 0; j < HALF; j += 16) {
-        float lf[16];
-        tmem_ld16(tmem + lanes + STASH + h * HALF + j, lf);
+        for (int k = 0; k < 4; ++k) slf[lane * 4 + (k ^ ((lane >> 1) & 3))] = lf[k];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const int eb = __shfl_sync(0xffffffffu, j < 32 ? ebl : ebh, (j + u) & 31);
-          const long long a = acc[j + u];
-          double d = scale_exp(i64_to_f64(a), a == 0 ? 0 : 9) + f32_to_f64(lf[u]);
-          d = d == 0.0 ? 0.0 : scale_exp(d, ea + eb);
-          if (P.alpha_neg) d = -d;
-          stg[lane * 16 + (u ^ (lane & 15))] = d;
-        }
+        for (int j = 0; j < COLS; j += 4)
+          if (j == 4 * seg) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sacc[lane * 4 + (k ^ ((lane >> 1) & 3))] = acc[j + k];
+          }
         __syncwarp();
-        const long n = nbase + j + col;
+        const int c = 4 * seg + col;
+        const int eb = __shfl_sync(0xffffffffu, ebl, c);
+        const long n = nbase + c;
         const bool col_ok = n < P.N && !skip;
         const long cno = col_ok ? (P.cn ? P.cn[n] : n) : 0;
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-          const int r = 2 * rr + hf;
-          double re = stg[(2 * r) * 16 + (col ^ ((2 * r) & 15))];
-          double im = stg[(2 * r + 1) * 16 + (col ^ ((2 * r + 1) & 15))];
+#pragma unroll 1
+        for (int rr = 0; rr < 2; ++rr) {
+          const int r = 8 * rr + hf;
           const long ro = __shfl_sync(0xffffffffu, roff, r);
+          const int e = __shfl_sync(0xffffffffu, ea, 2 * r) + eb;
+          double v[2];
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            const int at = (2 * r + w) * 4 + (col ^ (r & 3));
+            const long long x = sacc[at] - bias;
+            double d = f32_to_f64(slf[at]);
+            if (x != 0) d += scale_exp(i64_to_f64(x), 9 + u);
+            v[w] = scale_exp(d, e);
+            if (P.alpha_neg) v[w] = __hiloint2double(__double2hiint(v[w]) ^ 0x80000000, __double2loint(v[w]));
+          }
           if (!col_ok || mbase + r >= P.M) continue;
           double2 *o = P.C + ro + cno;
-          if (!P.alpha_p2) {
-            const double2 x = cmul(P.alpha, make_double2(re, im));
-            re = x.x;
-            im = x.y;
-          }
+          double2 y = make_double2(v[0], v[1]);
+          if (!P.alpha_p2) y = cmul(P.alpha, y);
           if (P.wmode == SW_ADD) {
-            atomicAdd(&o->x, re);
-            atomicAdd(&o->y, im);
+            atomicAdd(&o->x, y.x);
+            atomicAdd(&o->y, y.y);
           } else if (P.wmode == SW_STORE) {
-            *o = make_double2(re, im);
+            *o = y;
           } else {
-            *o = cadd(make_double2(re, im), cmul(P.beta, *o));
+            *o = cadd(y, cmul(P.beta, *o));
           }
         }
         __syncwarp();
@@ -450,7 +609,7 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
   }
   __syncthreads();
   if constexpr (PAIR) cluster_sync_all();
-  if (warp == 9) {
+  if (warp == EPI_WARPS + 1) {
     __syncwarp();
     tc_fence_after();
     tmem_dealloc<PAIR>(tmem, TMEM_COLS);
@@ -622,12 +781,12 @@ __global__ void __launch_bounds__(256) slice_pack_kernel(SideArgs a, SideArgs b,
   }
 }
 
-template <int STAGES, bool PAIR>
+template <int STAGES, bool PAIR>  // STAGES slots of SKB K blocks for each operand
 void launch_slices(SliceArgs &a, const SlicePlanes &A, const SlicePlanes &B, int units, int sms,
                    cudaStream_t st) {
-  constexpr int STAGE_BYTES = (BM + (PAIR ? SBN / 2 : SBN)) * ROW_BYTES;
-  constexpr int SMEM = STAGES * STAGE_BYTES + 256 + 8 * 4096 + 1024;
-  static_assert((2 * STAGES + 2 * NBUF + 1) * 8 + 8 <= 256, "barrier block");
+  constexpr int STAGE_BYTES = SKB * (BM + (PAIR ? SBN / 2 : SBN)) * ROW_BYTES;
+  constexpr int SMEM = STAGES * STAGE_BYTES + BAR_BYTES + EPI_WARPS * 1536 + 1024;
+  static_assert((4 * STAGES + 2 * NBUF + 1) * 8 + 8 <= BAR_BYTES, "barrier block");
   static_assert(SMEM <= 232448, "shared memory budget");
   auto kern = slice_gemm_kernel<STAGES, PAIR>;
   static const bool attr = [&] {
@@ -811,8 +970,8 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
     guard_beta = make_double2(1.0, 0.0);
   }
   const int u = static_cast<int>(units);
-  if (pair) launch_slices<8, true>(a, A, B, u, num_sms, st);
-  else launch_slices<6, false>(a, A, B, u, num_sms, st);
+  if (pair) launch_slices<4, true>(a, A, B, u, num_sms, st);
+  else launch_slices<3, false>(a, A, B, u, num_sms, st);
   // Inf or NaN in an operand: the FP64 kernel computes this product instead
   GemmDesc f = g.src;
   f.M = g.M;
