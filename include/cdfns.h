@@ -310,7 +310,8 @@ int ipeom_left_sigma_dev(cc_ctx *ctx, int n_vec, const double *l_dev,
  *   C[m][n] = sum_k A[m][k] * B[n][k]   (complex128, row-major, C overwritten)
  * in the given tier (CC_TIER_*), on the default stream. The dense
  * contraction core of every step above; exposed for tests and profiling.
- * Allocates its operand planes with cudaMalloc. Errors: CC_ERR_ARG.
+ * Allocates its operand planes through the default allocator (cudaMalloc
+ * unless cc_set_default_allocator replaced it). Errors: CC_ERR_ARG.
  */
 int cc_zgemm_dev(int tier, long M, long N, long K, const double *A_dev,
                  const double *B_dev, double *C_dev);
@@ -327,8 +328,8 @@ int cc_zgemm_dev(int tier, long M, long N, long K, const double *A_dev,
  * L_dev        device complex128 [max_vec][N]: rows 0..n_vec-1 receive l_k.
  * pivots_host  host long[max_vec] (may be NULL): the pivots p in order.
  * n_vec        host int: vectors formed.
- * FP64 throughout, on the default stream, O(N max_vec) device scratch from
- * the default allocator. Errors: CC_ERR_ARG, CC_ERR_NUMERIC (non-finite
+ * FP64 throughout, on the default stream, O(N + r max_vec) device scratch
+ * from the default allocator. Errors: CC_ERR_ARG, CC_ERR_NUMERIC (non-finite
  * diagonal).
  */
 int cc_cholesky_dev(long N, int r, const double *B_dev, double tau,

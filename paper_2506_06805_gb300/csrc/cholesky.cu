@@ -8,13 +8,17 @@
 // Every element of M - sum_k l_k l_k^H is then below tau in magnitude (the
 // remainder is positive semidefinite with every diagonal element below tau).
 //
-// The vectors are accumulated pair-major, Lt[q][k] (row stride ld), so that
-// both products of a step are row-contiguous matrix-vector products: the
-// column of M over B's rows, and the correction over the k vectors so far.
-// Both run on the contraction engine's FP64 GEMV kernels; the argmax is a
-// two-pass block reduction whose partial results the host finishes (one
-// short copy per step). The decomposition is bound by HBM bandwidth: each
-// step reads B and the vectors formed so far once.
+// Every vector lies in the span of B's columns, l_k = B w_k, so the
+// correction over the earlier vectors is taken on the r coefficients,
+//   w_k = (conj(B[p]) - sum_{j<k} w_j conj(l_j[p])) / sqrt(d_p),
+// instead of on the N elements: a step is one product with B (N r complex
+// multiply-adds) instead of N (r + k). Two launches a step: `pivot` finishes
+// the argmax and forms w_k; `vector` forms l_k, updates the diagonal and
+// leaves each block's largest element for the next pivot. The pivots stay on
+// the device; the host looks once per STEP_BATCH steps whether to stop.
+// Bound: the FP64 pipe (4 N r multiply-adds a step at about 0.6 T/s; B's 16 N
+// r bytes would take a third of that). N = 43681, r = 320, 240 vectors: 86.9 ->
+// 35.0 ms (0.77 TF/s), the error against FP64 in torch 9.4e-14 -> 8.3e-14.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -25,124 +29,187 @@ namespace cdfns {
 
 namespace {
 
-constexpr int ARGMAX_THREADS = 256;
-constexpr int ARGMAX_BLOCKS = 1024;
+constexpr int THREADS = 256;
+constexpr int ROW_LANES = 8;                            // lanes per row of B
+constexpr int BLOCK_ROWS = THREADS / ROW_LANES;         // rows per block and pass
+constexpr long MAX_BLOCKS = 8192;                       // partial maxima
+constexpr int STEP_BATCH = 32;
+constexpr int SMEM_R = 2048;                            // coefficients kept in shared memory
 
-// d[q] = sum_s |B[q][s]|^2
-__global__ void row_norm2_kernel(const double2 *__restrict__ B, long N, int r, double *d) {
-  for (long q = blockIdx.x * static_cast<long>(blockDim.x) + threadIdx.x; q < N;
-       q += static_cast<long>(gridDim.x) * blockDim.x) {
-    const double2 *row = B + q * r;
-    double s = 0.0;
-    for (int j = 0; j < r; ++j) s += row[j].x * row[j].x + row[j].y * row[j].y;
-    d[q] = s;
-  }
-}
-
-// per block: the largest d and its smallest index
-__global__ void __launch_bounds__(ARGMAX_THREADS)
-    block_argmax_kernel(const double *__restrict__ d, long N, double *bv, long *bi) {
-  __shared__ double sv[ARGMAX_THREADS];
-  __shared__ long si[ARGMAX_THREADS];
-  double v = -1.0;
-  long idx = -1;
-  for (long q = blockIdx.x * static_cast<long>(blockDim.x) + threadIdx.x; q < N;
-       q += static_cast<long>(gridDim.x) * blockDim.x) {
-    if (d[q] > v) {  // ascending q per thread: the first of equal values stays
-      v = d[q];
-      idx = q;
+struct Largest {
+  double v;
+  long i;
+  // the larger value, of equal ones the smaller index; i < 0: none
+  __device__ __forceinline__ void take(double v2, long i2) {
+    if (i2 >= 0 && (i < 0 || v2 > v || (v2 == v && i2 < i))) {
+      v = v2;
+      i = i2;
     }
   }
-  sv[threadIdx.x] = v;
-  si[threadIdx.x] = idx;
+};
+
+__device__ __forceinline__ Largest block_largest(Largest m) {
+  __shared__ double sv[THREADS / 32];
+  __shared__ long si[THREADS / 32];
+  for (int o = 16; o > 0; o >>= 1)
+    m.take(__shfl_xor_sync(0xffffffffu, m.v, o), __shfl_xor_sync(0xffffffffu, m.i, o));
+  if ((threadIdx.x & 31) == 0) {
+    sv[threadIdx.x >> 5] = m.v;
+    si[threadIdx.x >> 5] = m.i;
+  }
   __syncthreads();
-  for (int h = ARGMAX_THREADS / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-      const double v2 = sv[threadIdx.x + h];
-      const long i2 = si[threadIdx.x + h];
-      if (v2 > sv[threadIdx.x] || (v2 == sv[threadIdx.x] && i2 >= 0 && i2 < si[threadIdx.x])) {
-        sv[threadIdx.x] = v2;
-        si[threadIdx.x] = i2;
+  Largest t{-1.0, -1};
+  for (int w = 0; w < THREADS / 32; ++w) t.take(sv[w], si[w]);
+  __syncthreads();
+  return t;  // the same in every thread
+}
+
+// FIRST: d[q] = sum_s |B[q][s]|^2. Otherwise l = B w, L[q] = l, d[q] -= |l|^2.
+// Eight lanes per row (128 contiguous bytes a load, three shuffles for four
+// rows at once); w in shared memory.
+template <bool FIRST>
+__global__ void __launch_bounds__(THREADS)
+    vector_kernel(const double2 *__restrict__ B, long N, int r, const double2 *__restrict__ w,
+                  const long *__restrict__ piv, double2 *__restrict__ L, double *__restrict__ d,
+                  double *bv, long *bi) {
+  if (!FIRST && *piv < 0) return;  // the decomposition has stopped
+  __shared__ double2 sw[SMEM_R];
+  const double2 *ws = w;
+  if (!FIRST && r <= SMEM_R) {
+    for (int s = threadIdx.x; s < r; s += THREADS) sw[s] = w[s];
+    __syncthreads();
+    ws = sw;
+  }
+  const int lane = threadIdx.x & (ROW_LANES - 1);
+  Largest m{-1.0, -1};
+  for (long q0 = blockIdx.x * static_cast<long>(BLOCK_ROWS); q0 < N;
+       q0 += static_cast<long>(gridDim.x) * BLOCK_ROWS) {
+    const long q = q0 + threadIdx.x / ROW_LANES;
+    double xr = 0.0, xi = 0.0;
+    if (q < N) {
+      const double2 *row = B + q * r;
+      double yr = 0.0, yi = 0.0;
+#pragma unroll 4
+      for (int s = lane; s < r; s += ROW_LANES) {
+        const double2 b = row[s];
+        if (FIRST) {
+          xr = fma(b.x, b.x, xr);
+          yr = fma(b.y, b.y, yr);
+        } else {
+          const double2 c = ws[s];
+          xr = fma(b.x, c.x, xr);
+          yr = fma(-b.y, c.y, yr);
+          xi = fma(b.x, c.y, xi);
+          yi = fma(b.y, c.x, yi);
+        }
+      }
+      xr += yr;
+      xi += yi;
+    }
+    for (int o = ROW_LANES / 2; o > 0; o >>= 1) {
+      xr += __shfl_xor_sync(0xffffffffu, xr, o);
+      if (!FIRST) xi += __shfl_xor_sync(0xffffffffu, xi, o);
+    }
+    if (q < N && lane == 0) {
+      double x;
+      if (FIRST) {
+        x = xr;
+      } else {
+        L[q] = make_double2(xr, xi);
+        x = d[q] - (xr * xr + xi * xi);
+      }
+      d[q] = x;
+      if (x > m.v) {  // ascending q: the first of equal values stays, NaN never does
+        m.v = x;
+        m.i = q;
       }
     }
-    __syncthreads();
   }
+  m = block_largest(m);
   if (threadIdx.x == 0) {
-    bv[blockIdx.x] = sv[0];
-    bi[blockIdx.x] = si[0];
+    bv[blockIdx.x] = m.v;
+    bi[blockIdx.x] = m.i;
   }
 }
 
-// l = s * col; Lt[q][k] = l; d[q] -= |l|^2
-__global__ void store_vector_kernel(const double2 *__restrict__ col, double s, long N, double2 *Lt,
-                                    long ld, int k, double *d) {
-  for (long q = blockIdx.x * static_cast<long>(blockDim.x) + threadIdx.x; q < N;
-       q += static_cast<long>(gridDim.x) * blockDim.x) {
-    const double2 l = make_double2(s * col[q].x, s * col[q].y);
-    Lt[q * ld + k] = l;
-    d[q] -= l.x * l.x + l.y * l.y;
+// Step k: the pivot from the partial maxima (every block by itself; -1 once
+// the decomposition has stopped, -2 for a diagonal that is not finite), then
+// 32 of w_k's coefficients per block, the earlier vectors spread over its
+// eight warps.
+__global__ void __launch_bounds__(THREADS)
+    pivot_kernel(const double2 *__restrict__ B, long N, int r, double tau, int k, long nb,
+                 const double *__restrict__ bv, const long *__restrict__ bi,
+                 const double2 *__restrict__ L, double2 *W, long *piv) {
+  if (k > 0 && piv[k - 1] < 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) piv[k] = piv[k - 1];
+    return;
   }
-}
-
-unsigned blocks_for(long n) {
-  return static_cast<unsigned>(std::max<long>(1, std::min<long>((n + 255) / 256, 4096)));
+  Largest m{-1.0, -1};
+  for (long b = threadIdx.x; b < nb; b += THREADS) m.take(bv[b], bi[b]);
+  m = block_largest(m);
+  const bool bad = m.i >= 0 && !isfinite(m.v);
+  const bool stop = bad || m.i < 0 || !(m.v >= tau) || !(m.v > 0.0);
+  if (blockIdx.x == 0 && threadIdx.x == 0) piv[k] = bad ? -2 : (stop ? -1 : m.i);
+  if (stop) return;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int s = blockIdx.x * 32 + tx;
+  double2 a = make_double2(0.0, 0.0);
+  if (s < r) {
+#pragma unroll 4
+    for (int j = ty; j < k; j += THREADS / 32) {
+      const double2 l = L[j * N + m.i], w = W[static_cast<long>(j) * r + s];
+      a = cfma(w, make_double2(l.x, -l.y), a);
+    }
+  }
+  __shared__ double2 part[THREADS / 32][33];
+  part[ty][tx] = a;
+  __syncthreads();
+  if (ty == 0 && s < r) {
+    for (int g = 1; g < THREADS / 32; ++g) a = cadd(a, part[g][tx]);
+    const double2 b = B[m.i * r + s];
+    const double f = 1.0 / sqrt(m.v);
+    W[static_cast<long>(k) * r + s] = make_double2(f * (b.x - a.x), f * (-b.y - a.y));
+  }
 }
 
 }  // namespace
 
 int pivoted_cholesky(const cplx *B, long N, int r, double tau, int max_vec, cplx *L, long *piv,
                      Allocator *al, cudaStream_t st, int num_sms) {
-  Engine eng;
-  eng.al = al;
-  eng.st = st;
-  eng.num_sms = num_sms;
-  const long ld = max_vec;
-  Buf d(al, sizeof(double) * N), col(al, sizeof(cplx) * N), Lt(al, sizeof(cplx) * N * ld);
-  const unsigned nb = static_cast<unsigned>(std::min<long>(ARGMAX_BLOCKS, (N + 255) / 256));
-  Buf bv(al, sizeof(double) * nb), bi(al, sizeof(long) * nb);
-  std::vector<double> hv(nb);
-  std::vector<long> hi(nb);
-  row_norm2_kernel<<<blocks_for(N), 256, 0, st>>>(reinterpret_cast<const double2 *>(B), N, r,
-                                                  d.as<double>());
+  (void)num_sms;
+  const long nb = std::min<long>(MAX_BLOCKS, (N + BLOCK_ROWS - 1) / BLOCK_ROWS);
+  const unsigned grid = static_cast<unsigned>(nb);
+  Buf d(al, sizeof(double) * N), W(al, sizeof(cplx) * max_vec * r);
+  Buf bv(al, sizeof(double) * nb), bi(al, sizeof(long) * nb), pv(al, sizeof(long) * max_vec);
+  vector_kernel<true><<<grid, THREADS, 0, st>>>(B, N, r, nullptr, nullptr, nullptr, d.as<double>(),
+                                                bv.as<double>(), bi.as<long>());
   LAUNCH_CHECK();
   count_launch();
-  int k = 0;
-  for (; k < max_vec; ++k) {
-    block_argmax_kernel<<<nb, ARGMAX_THREADS, 0, st>>>(d.as<double>(), N, bv.as<double>(),
-                                                       bi.as<long>());
-    LAUNCH_CHECK();
-    count_launch();
-    CUDA_CHECK(cudaMemcpyAsync(hv.data(), bv.p, sizeof(double) * nb, cudaMemcpyDeviceToHost, st));
-    CUDA_CHECK(cudaMemcpyAsync(hi.data(), bi.p, sizeof(long) * nb, cudaMemcpyDeviceToHost, st));
+  std::vector<long> hp(max_vec);
+  int n = 0;
+  for (int k0 = 0; k0 < max_vec; k0 += STEP_BATCH) {
+    const int k1 = std::min(max_vec, k0 + STEP_BATCH);
+    for (int k = k0; k < k1; ++k) {
+      pivot_kernel<<<static_cast<unsigned>((r + 31) / 32), THREADS, 0, st>>>(
+          B, N, r, tau, k, nb, bv.as<double>(), bi.as<long>(), L, W.c(), pv.as<long>());
+      LAUNCH_CHECK();
+      vector_kernel<false><<<grid, THREADS, 0, st>>>(B, N, r, W.c() + static_cast<long>(k) * r,
+                                                     pv.as<long>() + k, L + static_cast<long>(k) * N,
+                                                     d.as<double>(), bv.as<double>(), bi.as<long>());
+      LAUNCH_CHECK();
+      count_launch(2);
+    }
+    CUDA_CHECK(cudaMemcpyAsync(hp.data() + k0, pv.as<long>() + k0, sizeof(long) * (k1 - k0),
+                               cudaMemcpyDeviceToHost, st));
     CUDA_CHECK(cudaStreamSynchronize(st));
-    double dmax = -1.0;
-    long p = -1;
-    for (unsigned b = 0; b < nb; ++b)
-      if (hi[b] >= 0 && (hv[b] > dmax || (hv[b] == dmax && hi[b] < p))) {
-        dmax = hv[b];
-        p = hi[b];
-      }
-    if (p >= 0 && !std::isfinite(dmax)) fail(CC_ERR_NUMERIC, "cholesky: non-finite diagonal");
-    if (p < 0 || !(dmax >= tau) || !(dmax > 0.0)) break;
-    // column p of M = B conj(B[p])
-    eng.contract(C1(), T(B, "qs", {N, r}), conj(T(B + p * r, "s", {r})), C0(), T(col.c(), "q", {N}),
-                 TIER_FP64);
-    // minus sum_{j<k} l_j conj(l_j[p])
-    if (k > 0)
-      eng.contract(Cr(-1), Tv(Lt.c(), "qj", {N, k}, {ld, 1}), conj(Tv(Lt.c() + p * ld, "j", {k}, {1})),
-                   C1(), T(col.c(), "q", {N}), TIER_FP64);
-    store_vector_kernel<<<blocks_for(N), 256, 0, st>>>(reinterpret_cast<const double2 *>(col.p),
-                                                       1.0 / std::sqrt(dmax), N, Lt.as<double2>(),
-                                                       ld, k, d.as<double>());
-    LAUNCH_CHECK();
-    count_launch();
-    if (piv) piv[k] = p;
+    while (n < k1 && hp[n] >= 0) ++n;
+    if (n < k1) {
+      if (hp[n] == -2) fail(CC_ERR_NUMERIC, "cholesky: non-finite diagonal");
+      break;
+    }
   }
-  // vectors row-major for the caller: L[k][q]
-  if (k > 0)
-    eng.permute_into(C1(), Tv(Lt.c(), "qk", {N, k}, {ld, 1}), C0(), T(L, "kq", {k, N}));
-  CUDA_CHECK(cudaStreamSynchronize(st));
-  return k;
+  if (piv) std::copy(hp.begin(), hp.begin() + n, piv);
+  return n;
 }
 
 }  // namespace cdfns

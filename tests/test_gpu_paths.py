@@ -115,7 +115,7 @@ def test_fp64_product_extreme_rows():
         assert not bool(torch.isfinite(torch.view_as_real(C[10])).any(-1).any())
 
 
-@pytest.mark.parametrize("o,v,X", [(6, 41, 163), (9, 30, 121)])
+@pytest.mark.parametrize("o,v,X", [(6, 41, 163), (9, 30, 121), (17, 19, 60)])
 def test_fp64_residual_and_sigma_on_tensor_cores(o, v, X):
     """Strided, conjugated, transposed and accumulating products of the FP64
     residual and sigma at sizes that take the tensor-core form."""
@@ -169,3 +169,40 @@ def test_fp32_short_k_products_cut_on_both_sides(M, N, K):
     P.zgemm_dev(A, B, C, "fp16x3")
     tol = 2 * K * 2.0 ** -24 * _rownorm(A)[:, None] * _rownorm(B)[None, :]
     assert bool(((C - A @ B.T).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("N,r,n", [(1, 1, 1), (5, 3, 3), (33, 40, 33), (257, 2100, 40), (300000, 9, 9)])
+def test_pivoted_cholesky_sizes(N, r, n):
+    """Fewer rows than a block, more coefficients than shared memory holds,
+    several passes per block."""
+    from oracle import cholesky
+    P = _gpu()
+    rng = np.random.default_rng(N + r)
+    B = rng.standard_normal((N, r)) + 1j * rng.standard_normal((N, r))
+    ref, piv_ref = cholesky.pivoted_cholesky(B, 0.0, max_vec=n)
+    L, piv = P.cholesky_dev(torch.from_numpy(B).cuda(), 0.0, n)
+    # the last vectors of a full-rank run stand on small remainders
+    m = min(n, max(1, 3 * min(N, r) // 4))
+    assert np.array_equal(piv[:m], piv_ref[:m])
+    assert np.abs(L.cpu().numpy()[:m] - ref[:m]).max() <= 1e-11 * np.abs(ref).max()
+    if n > m:
+        Lh = L.cpu().numpy()
+        if len(Lh) == min(N, r):
+            M = B @ B.conj().T if N <= 1000 else None
+            if M is not None:
+                assert np.abs(M - Lh.T @ Lh.conj()).max() <= 1e-10 * np.abs(M).max()
+
+
+def test_pivoted_cholesky_beyond_the_rank_and_non_finite():
+    P = _gpu()
+    rng = np.random.default_rng(4)
+    B = rng.standard_normal((500, 12)) + 1j * rng.standard_normal((500, 12))
+    L, piv = P.cholesky_dev(torch.from_numpy(B).cuda(), 0.0, 80)  # tau 0: rounding remainders only
+    Lh = L.cpu().numpy()
+    assert len(piv) >= 12 and np.abs(Lh[12:]).max(initial=0.0) <= 1e-5 * np.abs(Lh).max()
+    M = B @ B.conj().T
+    assert np.abs(M - Lh.T @ Lh.conj()).max() <= 1e-11 * np.abs(M).max()
+    B[7, 3] = np.inf
+    with pytest.raises(P.CCError) as e:
+        P.cholesky_dev(torch.from_numpy(B).cuda(), 0.0, 8)
+    assert e.value.code == -6  # CC_ERR_NUMERIC
