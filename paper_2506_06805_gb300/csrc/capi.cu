@@ -488,7 +488,13 @@ int cc_zgemm_dev(int tier, long M, long N, long K, const double *A, const double
   if (tier < CC_TIER_FP64 || tier > CC_TIER_FP16X3 || M < 1 || N < 1 || K < 1 || !A || !B || !C)
     return CC_ERR_ARG;
   return guarded(nullptr, [&] {
-    static cdfns::Allocator al;
+    // temporaries from the default allocator (a caching one turns the planes'
+    // cudaMalloc and cudaFree, which synchronise, into a lookup)
+    cdfns::Allocator al;
+    {
+      std::lock_guard<std::mutex> lk(cdfns::g_mu);
+      al = cdfns::g_default_alloc;
+    }
     cdfns::Engine eng;
     eng.al = &al;
     eng.st = cdfns::g_default_stream;
