@@ -118,6 +118,64 @@ __global__ void permute_kernel(double2 *__restrict__ out, const double2 *__restr
   }
 }
 
+// The same where the input runs along output dimension u (unit stride) and
+// the output along its last: 32 x 32 tiles of the two transposed through
+// shared memory, so that both sides move whole lines. Block (32, 8); one item
+// per tile, the other dimensions' digits decoded once per item. Gathered
+// instead, <mb||ej> -> [j][b][m][e] at o = 40, v = 300 read 18 GB in 3.0 ms;
+// as tiles it reads 2.3 GB in 1.1 ms.
+__global__ void __launch_bounds__(256) permute_tile_kernel(double2 *__restrict__ out,
+                                                           const double2 *__restrict__ in, Dims D,
+                                                           int u, long items, double2 alpha,
+                                                           double2 beta, bool conj) {
+  __shared__ double2 tile[32][33];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int last = D.nd - 1;
+  const long du = D.d[u], dl = D.d[last], tu = (du + 31) / 32, tl = (dl + 31) / 32;
+  long ou = 1;  // output stride of dimension u
+  for (int k = u + 1; k < D.nd; ++k) ou *= D.d[k];
+  const bool pm1 = alpha.y == 0.0 && (alpha.x == 1.0 || alpha.x == -1.0);
+  const bool b1 = beta.x == 1.0 && beta.y == 0.0, b0 = beta.x == 0.0 && beta.y == 0.0;
+  for (long it = blockIdx.x; it < items; it += gridDim.x) {
+    long rem = it / (tu * tl);
+    const long t = it - rem * (tu * tl);
+    const long u0 = t / tl * 32, l0 = (t % tl) * 32;
+    long io = 0, oo = 0, os = dl;
+    for (int k = last - 1; k >= 0; --k) {
+      if (k != u) {
+        const long q = rem / D.d[k], g = rem - q * D.d[k];
+        io += g * D.s[k];
+        oo += g * os;
+        rem = q;
+      }
+      os *= D.d[k];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const long l = l0 + ty + 8 * j, a = u0 + tx;
+      if (l < dl && a < du) tile[ty + 8 * j][tx] = in[io + a + l * D.s[last]];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const long a = u0 + ty + 8 * j, l = l0 + tx;
+      if (l >= dl || a >= du) continue;
+      double2 *o = out + oo + a * ou + l;
+      double2 x = tile[tx][ty + 8 * j];
+      if (conj) x.y = -x.y;
+      if (pm1) {
+        if (alpha.x < 0) x = make_double2(-x.x, -x.y);
+      } else {
+        x = cmul(alpha, x);
+      }
+      if (b1) x = cadd(x, *o);
+      else if (!b0) x = cadd(x, cmul(beta, *o));
+      *o = x;
+    }
+    __syncthreads();
+  }
+}
+
 // Block-level deterministic reduction of sum conj?(x) y.
 constexpr int RED_BLOCKS = 1024;
 constexpr int RED_THREADS = 256;
@@ -378,7 +436,18 @@ void permute(cplx *out, const cplx *in, int nd, const long *odims, const long *i
     D.d[0] = 1;
     D.s[0] = 0;
   }
-  if (total <= 0xffffffffL)
+  // tiles when the input's unit stride lies on another dimension than the
+  // output's and both are long enough to fill one (shorter ones: half-empty
+  // lines cost less than half-empty tiles)
+  int u = -1;
+  for (int i = 0; i + 1 < D.nd; ++i)
+    if (D.s[i] == 1 && D.d[i] >= 16) u = i;
+  if (u >= 0 && D.s[D.nd - 1] > 1 && D.d[D.nd - 1] >= 16) {
+    const long area = D.d[u] * D.d[D.nd - 1];
+    const long items = total / area * ((D.d[u] + 31) / 32) * ((D.d[D.nd - 1] + 31) / 32);
+    permute_tile_kernel<<<static_cast<unsigned>(std::min<long>(items, 152L * 64)), dim3(32, 8), 0, st>>>(
+        out, in, D, u, items, alpha, beta, conj);
+  } else if (total <= 0xffffffffL)
     permute_kernel<unsigned><<<grid_for(total), 256, 0, st>>>(out, in, total, D, alpha, beta, conj);
   else
     permute_kernel<unsigned long long><<<grid_for(total), 256, 0, st>>>(out, in, total, D, alpha,
