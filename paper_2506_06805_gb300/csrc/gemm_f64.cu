@@ -223,72 +223,117 @@ __global__ void gemv_kt_kernel(long N, long K, const double2 *__restrict__ A,
   }
 }
 
-// Same contraction with one warp per output element and the lanes striding
-// k: coalesced when the operand's innermost K index has unit stride.
-template <bool F32>
-__global__ void gemv_warp_kernel(long N, long K, const double2 *__restrict__ A,
-                                 const long *__restrict__ ak, bool conjA,
-                                 const double2 *__restrict__ B, const long *__restrict__ bn,
-                                 const long *__restrict__ bk, long ldb, bool conjB, double2 *C,
-                                 const long *__restrict__ cn, long ldc, double2 alpha,
-                                 double2 beta) {
-  const int lane = threadIdx.x & 31;
-  const long wpb = blockDim.x >> 5;
-  for (long n = blockIdx.x * wpb + (threadIdx.x >> 5); n < N; n += static_cast<long>(gridDim.x) * wpb) {
-    const long bo = bn ? bn[n] : n * ldb;
-    // four independent loads per lane in flight (offset tables resolve first)
-    double2 ac[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
-                     make_double2(0.0, 0.0)};
-    long k = lane;
-    if (F32) {
-      // runs of 4 x 4 products per lane in FP32, each run added in FP64
-      for (; k + 96 < K; k += 128) {
-        float xr = 0.f, xi = 0.f;
+// Same contraction with a warp per output element and the lanes striding k:
+// coalesced when the operand's innermost K index has unit stride. Blocks of
+// 128 k per step; F32: a lane's four products of a block in FP32, that run
+// added in FP64.
+//   R > 1: R outputs per warp, whose vector elements, table entries and
+//   conversions are shared (many outputs: a warp each was bound by those,
+//   2.4 TB/s at 12000 x 12000). W > 1: the blocks of one output dealt to the
+//   W warps of the thread block (few outputs: 320 x 12000 ran on 320 warps).
+// Neither changes the FP32 runs. 12000 x 12000 (FP32) 952 -> 557 us, 320 x
+// 12000 (FP64) 120 -> 71 us, 1600 x 12000 (FP32) 310 -> 97 us.
+template <bool F32, int R, int W>
+__global__ void __launch_bounds__(256) gemv_warp_kernel(long N, long K, const double2 *__restrict__ A,
+                                                        const long *__restrict__ ak, bool conjA,
+                                                        const double2 *__restrict__ B,
+                                                        const long *__restrict__ bn,
+                                                        const long *__restrict__ bk, long ldb,
+                                                        bool conjB, double2 *C,
+                                                        const long *__restrict__ cn, long ldc,
+                                                        double2 alpha, double2 beta) {
+  static_assert(W == 1 || (W == 8 && R == 1), "one output per block, or whole warps");
+  __shared__ double2 part[W];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int kw = W == 1 ? 0 : warp;  // first block of this warp
+  const long g0 = W == 1 ? blockIdx.x * 8L + warp : blockIdx.x;
+  const long gstep = W == 1 ? static_cast<long>(gridDim.x) * 8 : gridDim.x;
+  for (long n0 = g0 * R; n0 < N; n0 += gstep * R) {
+    const double2 *row[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const long n = min(n0 + r, N - 1);
+      row[r] = B + (bn ? bn[n] : n * ldb);
+    }
+    double2 ac[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) ac[r] = make_double2(0.0, 0.0);
+    for (long k0 = 128L * kw; k0 < K; k0 += 128L * W) {
+      long k = k0 + lane;
+      if (k + 96 < K) {
+        long ib[4];
+        double2 av[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const long kk = k + 32 * u;
-          cfma32(A[ak ? ak[kk] : kk], B[bo + (bk ? bk[kk] : kk)], conjA, conjB, xr, xi);
+          av[u] = A[ak ? ak[kk] : kk];
+          ib[u] = bk ? bk[kk] : kk;
         }
-        ac[0].x += f32_to_f64(xr);
-        ac[0].y += f32_to_f64(xi);
-      }
-    }
-    for (; k + 96 < K; k += 128) {
-      long ia[4], ib[4];
+        if (F32) {
+          float2 a[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        ia[u] = ak ? ak[k + 32 * u] : k + 32 * u;
-        ib[u] = bo + (bk ? bk[k + 32 * u] : k + 32 * u);
-      }
-      double2 a[4], b[4];
+          for (int u = 0; u < 4; ++u)
+            a[u] = make_float2(f64_to_f32(av[u].x), conjA ? -f64_to_f32(av[u].y) : f64_to_f32(av[u].y));
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = A[ia[u]];
-        b[u] = B[ib[u]];
-      }
+          for (int r = 0; r < R; ++r) {
+            double2 b[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (conjA) a[u].y = -a[u].y;
-        if (conjB) b[u].y = -b[u].y;
-        ac[u] = cfma(a[u], b[u], ac[u]);
+            for (int u = 0; u < 4; ++u) b[u] = row[r][ib[u]];
+            float xr = 0.f, xi = 0.f;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const float br = f64_to_f32(b[u].x), bi = conjB ? -f64_to_f32(b[u].y) : f64_to_f32(b[u].y);
+              xr = fmaf(a[u].x, br, fmaf(-a[u].y, bi, xr));
+              xi = fmaf(a[u].x, bi, fmaf(a[u].y, br, xi));
+            }
+            ac[r].x += f32_to_f64(xr);
+            ac[r].y += f32_to_f64(xi);
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              double2 a = av[u], b = row[r][ib[u]];
+              if (conjA) a.y = -a.y;
+              if (conjB) b.y = -b.y;
+              ac[r] = cfma(a, b, ac[r]);
+            }
+        }
+      } else {
+        for (; k < K; k += 32) {
+          double2 a = A[ak ? ak[k] : k];
+          if (conjA) a.y = -a.y;
+          const long ib = bk ? bk[k] : k;
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            double2 b = row[r][ib];
+            if (conjB) b.y = -b.y;
+            ac[r] = cfma(a, b, ac[r]);
+          }
+        }
       }
     }
-    for (; k < K; k += 32) {
-      double2 a = A[ak ? ak[k] : k];
-      double2 b = B[bo + (bk ? bk[k] : k)];
-      if (conjA) a.y = -a.y;
-      if (conjB) b.y = -b.y;
-      ac[0] = cfma(a, b, ac[0]);
-    }
-    double2 acc = cadd(cadd(ac[0], ac[1]), cadd(ac[2], ac[3]));
-    for (int o = 16; o > 0; o >>= 1) {
-      acc.x += __shfl_down_sync(0xffffffffu, acc.x, o);
-      acc.y += __shfl_down_sync(0xffffffffu, acc.y, o);
-    }
-    if (lane == 0) {
-      const long off = cn ? cn[n] : n * ldc;
-      const double2 x = cmul(alpha, acc);
-      C[off] = (beta.x == 0.0 && beta.y == 0.0) ? x : cadd(x, cmul(beta, C[off]));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      double2 acc = ac[r];
+      for (int o = 16; o > 0; o >>= 1) {
+        acc.x += __shfl_down_sync(0xffffffffu, acc.x, o);
+        acc.y += __shfl_down_sync(0xffffffffu, acc.y, o);
+      }
+      if (W > 1) {
+        if (lane == 0) part[warp] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0)
+          for (int w = 1; w < W; ++w) acc = cadd(acc, part[w]);
+        __syncthreads();
+      }
+      if (lane == 0 && (W == 1 || warp == 0) && n0 + r < N) {
+        const long n = n0 + r;
+        const long off = cn ? cn[n] : n * ldc;
+        const double2 x = cmul(alpha, acc);
+        C[off] = (beta.x == 0.0 && beta.y == 0.0) ? x : cadd(x, cmul(beta, C[off]));
+      }
     }
   }
 }
@@ -385,8 +430,14 @@ void gemm_f64(const GemmDesc &g, cudaStream_t st, int num_sms) {
   if (rowvec || colvec) {
     const long n_out = rowvec ? g.N : g.M;
     if (g.k_contig) {
-      const unsigned wb = static_cast<unsigned>(std::min<long>((n_out + 7) / 8, 65535));
-      auto kern = g.f32 ? gemv_warp_kernel<true> : gemv_warp_kernel<false>;
+      // a block per output below 16 warps per SM; four outputs a warp while
+      // that still leaves 16; a warp per output between
+      const bool few = n_out < 16L * num_sms && g.K >= 1024, many = n_out >= 64L * num_sms;
+      const long per_block = few ? 1 : (many ? 32 : 8);
+      const unsigned wb = static_cast<unsigned>(std::min<long>((n_out + per_block - 1) / per_block, 65535));
+      auto kern = few    ? (g.f32 ? gemv_warp_kernel<true, 1, 8> : gemv_warp_kernel<false, 1, 8>)
+                  : many ? (g.f32 ? gemv_warp_kernel<true, 4, 1> : gemv_warp_kernel<false, 4, 1>)
+                         : (g.f32 ? gemv_warp_kernel<true, 1, 1> : gemv_warp_kernel<false, 1, 1>);
       if (rowvec)
         kern<<<wb, 256, 0, st>>>(n_out, g.K, g.A, g.ak, g.conjA, g.B, g.bn, g.bk, g.ldb, g.conjB,
                                  g.C, g.cn, 1, g.alpha, g.beta);

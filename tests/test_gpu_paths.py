@@ -206,3 +206,17 @@ def test_pivoted_cholesky_beyond_the_rank_and_non_finite():
     with pytest.raises(P.CCError) as e:
         P.cholesky_dev(torch.from_numpy(B).cuda(), 0.0, 8)
     assert e.value.code == -6  # CC_ERR_NUMERIC
+
+
+@pytest.mark.parametrize("n,K", [(1, 5000), (1, 129), (320, 12001), (2432, 1024), (2431, 1023),
+                                 (9729, 131), (12000, 300)])
+@pytest.mark.parametrize("side", ["row", "column"])
+def test_fp64_matrix_vector(n, K, side):
+    """A block, a warp or a quarter of a warp per output, with remainders."""
+    P = _gpu()
+    g = torch.Generator(device="cuda").manual_seed(n + K)
+    V, x = _cn(g, n, K), _cn(g, 1, K)
+    A, B = (x, V) if side == "row" else (V, x)
+    C = torch.empty((A.shape[0], B.shape[0]), dtype=torch.complex128, device="cuda")
+    P.zgemm_dev(A, B, C, "fp64")
+    _check_product(A, B, C)
