@@ -739,24 +739,6 @@ __global__ void ip_unpack_kernel(const double2 *vec, int k, int o, int v, double
   }
 }
 
-__global__ void ip_pack_kernel(const double2 *r1, const double2 *r2, int k, int o, int v,
-                               double2 *vec) {
-  const long np = static_cast<long>(o) * (o - 1) / 2;
-  const long dim = o + np * v;
-  GRID_STRIDE(idx, static_cast<long>(k) * dim) {
-    const long kk = idx / dim, rem = idx % dim;
-    if (rem < o) {
-      vec[idx] = r1[kk * o + rem];
-    } else {
-      const long q = rem - o;
-      int i, j;
-      pair_decode(q / v, o, &i, &j);
-      const int b = static_cast<int>(q % v);
-      vec[idx] = r2[((kk * o + i) * o + j) * v + b];
-    }
-  }
-}
-
 __global__ void ip_diag_kernel(const double2 *Hoo, const double2 *Hvv, int o, int v, double2 *d) {
   const long np = static_cast<long>(o) * (o - 1) / 2;
   const long dim = o + np * v;
@@ -774,36 +756,44 @@ __global__ void ip_diag_kernel(const double2 *Hoo, const double2 *Hvv, int o, in
   }
 }
 
-__global__ void ip_diag_apply_kernel(const double2 *r1, const double2 *r2, const double2 *doo,
-                                     const double2 *dvv, int k, int o, int v, double2 *s1,
-                                     double2 *s2) {
-  const long per = static_cast<long>(o) * o * v;
-  GRID_STRIDE(idx, static_cast<long>(k) * per) {
-    const long kk = idx / per, rem = idx % per;
-    const int b = static_cast<int>(rem % v);
-    const int j = static_cast<int>((rem / v) % o);
-    const int i = static_cast<int>(rem / (static_cast<long>(v) * o));
-    const double2 d = csub(csub(dvv[b], doo[i]), doo[j]);
-    s2[idx] = cadd(s2[idx], cmul(d, r2[idx]));
-    if (rem < o) s1[kk * o + rem] = csub(s1[kk * o + rem], cmul(doo[rem], r1[kk * o + rem]));
-  }
-}
-
-// s2 += tA + tB + tC - P(ij) X1 + P(ij) X2 on [k][o][o][v] tensors
-__global__ void sigma_combine_kernel(double2 *s2, const double2 *tA, const double2 *tB,
-                                     const double2 *tC, const double2 *X1, const double2 *X2, int k,
-                                     int o, int v) {
-  const long per = static_cast<long>(o) * o * v;
-  GRID_STRIDE(idx, static_cast<long>(k) * per) {
-    const long kk = idx / per, rem = idx % per;
-    const int b = static_cast<int>(rem % v);
-    const int j = static_cast<int>((rem / v) % o);
-    const int i = static_cast<int>(rem / (static_cast<long>(v) * o));
-    const long sw = kk * per + (static_cast<long>(j) * o + i) * v + b;
-    double2 x = cadd(cadd(s2[idx], tA[idx]), cadd(tB[idx], tC[idx]));
-    x = cadd(x, csub(X1[sw], X1[idx]));
-    x = cadd(x, csub(X2[idx], X2[sw]));
-    s2[idx] = x;
+// The last step of a sigma build, straight into the packed vectors
+// [k][o + o(o-1)/2 v]: the two-body terms summed, the exact one-body diagonal
+// added (FP64), only i < j computed and only the unique elements written.
+//   right: s2 + tA + tB + tC - P(ij) X1 + P(ij) X2 + (d_b - d_i - d_j) r2
+//   left:  G - G(i<->j) + (d_b - d_i - d_j) r2, with G in tA
+//   1h:    s1 - d_i r1
+// One warp per (vector, pair), lanes along b. As three passes (combine,
+// diagonal, pack) over the full [k][o][o][v] tensors it took 245 us for eight
+// vectors at o = 40, v = 300; FINISH_FIGURES, where the FP64 additions (two a
+// clock and SM) bound it.
+template <bool LEFT>
+__global__ void __launch_bounds__(256) sigma_finish_kernel(
+    const double2 *__restrict__ s1, const double2 *__restrict__ s2, const double2 *__restrict__ tA,
+    const double2 *__restrict__ tB, const double2 *__restrict__ tC, const double2 *__restrict__ X1,
+    const double2 *__restrict__ X2, const double2 *__restrict__ r1, const double2 *__restrict__ r2,
+    const double2 *__restrict__ doo, const double2 *__restrict__ dvv, int o, int v, double2 *vec) {
+  const long np = static_cast<long>(o) * (o - 1) / 2, dim = o + np * v;
+  const long kk = blockIdx.y;
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < o; i += blockDim.x)
+      vec[kk * dim + i] = csub(s1[kk * o + i], cmul(doo[i], r1[kk * o + i]));
+  const long p = blockIdx.x * 8L + (threadIdx.x >> 5);
+  if (p >= np) return;
+  int i, j;
+  pair_decode(p, o, &i, &j);
+  const long ij = ((kk * o + i) * o + j) * v, ji = ((kk * o + j) * o + i) * v;
+  const double2 di = doo[i], dj = doo[j];
+  double2 *out = vec + kk * dim + o + p * v;
+  for (int b = threadIdx.x & 31; b < v; b += 32) {
+    double2 x;
+    if (LEFT) {
+      x = csub(tA[ij + b], tA[ji + b]);
+    } else {
+      x = cadd(cadd(s2[ij + b], tA[ij + b]), cadd(tB[ij + b], tC[ij + b]));
+      x = cadd(x, csub(X1[ji + b], X1[ij + b]));
+      x = cadd(x, csub(X2[ij + b], X2[ji + b]));
+    }
+    out[b] = cadd(x, cmul(csub(csub(dvv[b], di), dj), r2[ij + b]));
   }
 }
 
@@ -1151,13 +1141,6 @@ void ip_unpack(const cplx *vec, int k, int o, int v, cplx *r1, cplx *r2, cudaStr
   count_launch();
 }
 
-void ip_pack(const cplx *r1, const cplx *r2, int k, int o, int v, cplx *vec, cudaStream_t st) {
-  const long dim = o + static_cast<long>(o) * (o - 1) / 2 * v;
-  ip_pack_kernel<<<grid_for(k * dim), 256, 0, st>>>(r1, r2, k, o, v, vec);
-  LAUNCH_CHECK();
-  count_launch();
-}
-
 void ip_diag(const cplx *Hoo, const cplx *Hvv, int o, int v, cplx *d, cudaStream_t st) {
   const long dim = o + static_cast<long>(o) * (o - 1) / 2 * v;
   ip_diag_kernel<<<grid_for(dim), 256, 0, st>>>(Hoo, Hvv, o, v, d);
@@ -1165,20 +1148,25 @@ void ip_diag(const cplx *Hoo, const cplx *Hvv, int o, int v, cplx *d, cudaStream
   count_launch();
 }
 
-void ip_diag_apply(const cplx *r1, const cplx *r2, const cplx *doo, const cplx *dvv, int k, int o,
-                   int v, cplx *s1, cplx *s2, cudaStream_t st) {
-  ip_diag_apply_kernel<<<grid_for(static_cast<long>(k) * o * o * v), 256, 0, st>>>(r1, r2, doo, dvv, k,
-                                                                                  o, v, s1, s2);
-  LAUNCH_CHECK();
-  count_launch();
-}
-
-void sigma_combine(cplx *s2, const cplx *tA, const cplx *tB, const cplx *tC, const cplx *X1,
-                   const cplx *X2, int k, int o, int v, cudaStream_t st) {
-  sigma_combine_kernel<<<grid_for(static_cast<long>(k) * o * o * v), 256, 0, st>>>(s2, tA, tB, tC, X1,
-                                                                                  X2, k, o, v);
-  LAUNCH_CHECK();
-  count_launch();
+void sigma_finish(const cplx *s1, const cplx *s2, const cplx *tA, const cplx *tB, const cplx *tC,
+                  const cplx *X1, const cplx *X2, const cplx *r1, const cplx *r2, const cplx *doo,
+                  const cplx *dvv, int k, int o, int v, cplx *vec, cudaStream_t st) {
+  const long np = static_cast<long>(o) * (o - 1) / 2;
+  for (int k0 = 0; k0 < k; k0 += 65535) {  // the grid's y extent
+    const long n1 = static_cast<long>(k0) * o, n2 = n1 * o * v, nv = k0 * (o + np * v);
+    const dim3 grid(static_cast<unsigned>(std::max<long>(1, (np + 7) / 8)),
+                    static_cast<unsigned>(std::min(k - k0, 65535)));
+    if (s2)
+      sigma_finish_kernel<false><<<grid, 256, 0, st>>>(s1 + n1, s2 + n2, tA + n2, tB + n2, tC + n2,
+                                                       X1 + n2, X2 + n2, r1 + n1, r2 + n2, doo, dvv,
+                                                       o, v, vec + nv);
+    else
+      sigma_finish_kernel<true><<<grid, 256, 0, st>>>(s1 + n1, nullptr, tA + n2, nullptr, nullptr,
+                                                      nullptr, nullptr, r1 + n1, r2 + n2, doo, dvv,
+                                                      o, v, vec + nv);
+    LAUNCH_CHECK();
+    count_launch();
+  }
 }
 
 void split_diag(const cplx *A, int n, cplx *off, cplx *diag, cudaStream_t st) {

@@ -86,16 +86,15 @@ void make_pairs(int n, int *pi, int *pj, cudaStream_t st);
 // --- IP vectors --------------------------------------------------------------------
 // packed [k][o + npair*v] <-> r1 [k][o], r2 [k][o][o][v] (antisymmetric)
 void ip_unpack(const cplx *vec, int k, int o, int v, cplx *r1, cplx *r2, cudaStream_t st);
-void ip_pack(const cplx *r1, const cplx *r2, int k, int o, int v, cplx *vec, cudaStream_t st);
 // d[o + pairs*v]: -Hoo_ii and Hvv_bb - Hoo_ii - Hoo_jj
 void ip_diag(const cplx *Hoo, const cplx *Hvv, int o, int v, cplx *d, cudaStream_t st);
-// s2[K][i][j][b] += (dvv_b - doo_i - doo_j) r2, s1[K][i] -= doo_i r1 (the
-// diagonal one-body part of sigma, exact in FP64)
-void ip_diag_apply(const cplx *r1, const cplx *r2, const cplx *doo, const cplx *dvv, int k, int o,
-                   int v, cplx *s1, cplx *s2, cudaStream_t st);
-// s2 += tA + tB + tC - (X1 - X1(i<->j)) + (X2 - X2(i<->j)), [k][o][o][v]
-void sigma_combine(cplx *s2, const cplx *tA, const cplx *tB, const cplx *tC, const cplx *X1,
-                   const cplx *X2, int k, int o, int v, cudaStream_t st);
+// packed vec [k][o + npair*v] from the parts of a sigma build: s2 + tA + tB +
+// tC - (X1 - X1(i<->j)) + (X2 - X2(i<->j)), or tA - tA(i<->j) when s2 is NULL
+// (left sigma), each [k][o][o][v], plus (dvv_b - doo_i - doo_j) r2; and
+// s1 - doo_i r1 (the diagonal one-body part, exact in FP64)
+void sigma_finish(const cplx *s1, const cplx *s2, const cplx *tA, const cplx *tB, const cplx *tC,
+                  const cplx *X1, const cplx *X2, const cplx *r1, const cplx *r2, const cplx *doo,
+                  const cplx *dvv, int k, int o, int v, cplx *vec, cudaStream_t st);
 // off = A with zero diagonal, diag = diagonal of A (n x n)
 void split_diag(const cplx *A, int n, cplx *off, cplx *diag, cudaStream_t st);
 // x[r] = R[r] / (w[r] - d) with |den| floored at 1e-8

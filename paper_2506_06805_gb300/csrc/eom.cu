@@ -163,9 +163,8 @@ void sigma_body(std::vector<Ctx *> &sys, const std::vector<int> &k, cudaStream_t
     const int kk = k[q];
     if (kk == 0) continue;
     auto &w = c.sws;
-    sigma_combine(w.s2.c(), w.tA.c(), w.tB.c(), w.tC.c(), w.X1.c(), w.X2.c(), kk, c.o, c.v, st);
-    ip_diag_apply(w.r1.c(), w.r2.c(), c.doo.c(), c.dvv.c(), kk, c.o, c.v, w.s1.c(), w.s2.c(), st);
-    ip_pack(w.s1.c(), w.s2.c(), kk, c.o, c.v, w.sout.c(), st);
+    sigma_finish(w.s1.c(), w.s2.c(), w.tA.c(), w.tB.c(), w.tC.c(), w.X1.c(), w.X2.c(), w.r1.c(),
+                 w.r2.c(), c.doo.c(), c.dvv.c(), kk, c.o, c.v, w.sout.c(), st);
   }
 }
 
@@ -297,7 +296,6 @@ void left_sigma_body(Ctx &c, int kk, const cplx *lin, cplx *sout) {
   auto L2 = [&](const char *ix) { return T(w.r2.c(), ix, {kk, o, o, v}); };
   auto G = [&](const char *ix) { return T(w.tA.c(), ix, {kk, o, o, v}); };
   auto S1 = [&](const char *ix) { return T(w.s1.c(), ix, {kk, o}); };
-  auto S2 = [&](const char *ix) { return T(w.s2.c(), ix, {kk, o, o, v}); };
   ip_unpack(lin, kk, o, v, w.r1.c(), w.r2.c(), st);
   // 1h: -sum_i H_mi l_i - 1/2 sum_bij H_mbij l_ij^b
   c.eng.contract(Cr(-1), L1("Ki"), T(c.Hoo_off.c(), "mi", {o, o}), C0(), S1("Km"), TIER_FP64);
@@ -318,10 +316,8 @@ void left_sigma_body(Ctx &c, int kk, const cplx *lin, cplx *sout) {
                  T(w.xe.c(), "Ke", {kk, v}), tr);
   c.eng.contract(Cr(-0.5), T(w.xe.c(), "Ke", {kk, v}), stable(T(c.oovv.c(), "mnef", {o, o, v, v})),
                  C1(), G("Kmnf"), tr);
-  c.eng.permute_into(C1(), G("Kijb"), C0(), S2("Kijb"));
-  c.eng.permute_into(Cr(-1), G("Kjib"), C1(), S2("Kijb"));
-  ip_diag_apply(w.r1.c(), w.r2.c(), c.doo.c(), c.dvv.c(), kk, o, v, w.s1.c(), w.s2.c(), st);
-  ip_pack(w.s1.c(), w.s2.c(), kk, o, v, sout, st);
+  sigma_finish(w.s1.c(), nullptr, w.tA.c(), nullptr, nullptr, nullptr, nullptr, w.r1.c(), w.r2.c(),
+               c.doo.c(), c.dvv.c(), kk, o, v, sout, st);
 }
 
 }  // namespace
