@@ -504,18 +504,20 @@ void Engine::product_f64(const GemmDesc &g, bool a_rows, bool b_rows) {
   gemm_f64(g, st, num_sms);
 }
 
-size_t Engine::slice_budget(int which) {
+size_t Engine::slice_budget(int which, size_t need) {
   const auto it = planes_.find(which);
   const size_t held = it == planes_.end() ? 0 : it->second.bytes;
+  if (held >= need) return held;  // (no query of the device, as in a captured pass)
   return std::max(held, std::min(SLICE_BUDGET, device_avail(al) / 8));
 }
 
 bool Engine::run_slices(const GemmDesc &g, bool a_rows, bool b_rows) {
   // a capped context keeps the memory its cap was chosen for
   if (al->limit) return false;
-  const size_t cap_a = slice_budget(SLICE_SLOT_A), cap_b = slice_budget(SLICE_SLOT_B);
   // K blocks keep the integer sums of a tile within their range
   const long kb = std::min<long>(g.K, 65536);
+  const size_t cap_a = slice_budget(SLICE_SLOT_A, slice_bytes(true, g.M, kb)),
+               cap_b = slice_budget(SLICE_SLOT_B, slice_bytes(false, g.N, kb));
   auto rows_in = [&](bool a_side, size_t cap, long rows) {
     if (slice_bytes(a_side, rows, kb) <= cap) return rows;
     const size_t per = slice_bytes(a_side, 1024, kb) / 1024 + 1;

@@ -107,7 +107,7 @@ class Engine {
   // Device bytes each operand's digit planes of an FP64 product may take:
   // what is already held in their slot, or up to an eighth of the room left
   // and SLICE_BUDGET
-  size_t slice_budget(int which);
+  size_t slice_budget(int which, size_t need);
   static constexpr size_t SLICE_BUDGET = size_t(4) << 30;
   static constexpr int SLICE_SLOT_A = 1000, SLICE_SLOT_B = 1001;
   void clear_cache() {

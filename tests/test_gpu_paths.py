@@ -220,3 +220,17 @@ def test_fp64_matrix_vector(n, K, side):
     C = torch.empty((A.shape[0], B.shape[0]), dtype=torch.complex128, device="cuda")
     P.zgemm_dev(A, B, C, "fp64")
     _check_product(A, B, C)
+
+
+def test_fp64_solve_on_tensor_cores_with_and_without_graphs():
+    """The captured sigma replays the digit-plane products (their planes are
+    part of the graph's key); FP64 to the last steps of the Davidson."""
+    P = _gpu()
+    eps, L = synth.make_system(9, 41, 163, seed=8)
+    roots = []
+    for graphs in (True, False):
+        with P.System(eps, 3 * L, n_occ=9, tier="fp64", eom_tier="fp64") as s:
+            s.set_graphs(graphs)
+            s.ccsd(tol=1e-10)
+            roots.append(s.ipeom(4, tol=1e-9)[0])
+    assert np.abs(np.sort_complex(roots[0]) - np.sort_complex(roots[1])).max() <= 1e-10
