@@ -488,8 +488,11 @@ int cc_zgemm_dev(int tier, long M, long N, long K, const double *A, const double
   if (tier < CC_TIER_FP64 || tier > CC_TIER_FP16X3 || M < 1 || N < 1 || K < 1 || !A || !B || !C)
     return CC_ERR_ARG;
   return guarded(nullptr, [&] {
-    // temporaries from the default allocator (a caching one turns the planes'
-    // cudaMalloc and cudaFree, which synchronise, into a lookup)
+    // Temporaries from the default allocator: a caching one turns the planes'
+    // cudaMalloc and cudaFree, which synchronise, into a lookup. Per call, with
+    // torch's allocator / with cudaMalloc: FP16 209 x 171 x 222 83 / 204 us (74
+    // where the driver holds free pages from earlier blocks), FP64
+    // 209 x 171 x 222 130 / 297, 1536 x 1000 x 1200 560 / 870.
     cdfns::Allocator al;
     {
       std::lock_guard<std::mutex> lk(cdfns::g_mu);

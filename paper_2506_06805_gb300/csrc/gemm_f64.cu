@@ -1,4 +1,4 @@
-// Complex FP64 GEMM on the FP64 pipe (the plain CC_TIER_FP64 path).
+// Complex FP64 GEMM on the FP64 pipe (FP64 products too small for digit planes).
 //
 // C(m, n) = alpha * sum_k A(m, k) B(n, k) + beta * C(m, n) with operands
 // gathered through offset tables (see GemmDesc). 64 x 64 complex output tile

@@ -24,8 +24,8 @@
 // 2.7e-18 / 6.0e-18, K = 20000 1.1e-18 / 4.3e-18.
 //
 // Measured against the FP64 kernels: product of 1536 x 1000 x 1200 14.7 ->
-// 0.88 ms, ladder at o = 15, v = 131, X = 517 983 -> 22 ms, FP64 residual at
-// o = 12, v = 72, X = 288 80.7 -> 5.3 ms.
+// 0.57 ms, ladder at o = 15, v = 131, X = 517 983 -> 21 ms, FP64 residual at
+// o = 12, v = 72, X = 288 80.7 -> 5.1 ms.
 //
 // Rows that hold an Inf or NaN cannot be cut: the packing raises a flag on
 // the device, the slice kernel then stores nothing, and a guarded launch of
