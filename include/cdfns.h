@@ -48,8 +48,14 @@ extern "C" {
 /* Precision tiers of the contractions (cc_set_precision). Control steps
  * (denominators, DIIS, energies, norms, Davidson subspace) are FP64 in
  * every tier. */
-#define CC_TIER_FP64 0   /* FP64: exact digit products on the tensor cores
-                          * where they pay, else the FP64 pipe */
+#define CC_TIER_FP64 0   /* FP64: large products as sums of integer digit
+                          * products on the tensor cores, others (and all of
+                          * a context with a memory limit) on the FP64 pipe.
+                          * Either way the error of an element is that of an
+                          * FP64 sum of its terms: elements for which the
+                          * digits, cut relative to the largest magnitudes of
+                          * the two rows, would give less are computed on the
+                          * FP64 pipe */
 #define CC_TIER_TF32 1   /* tcgen05 kind::tf32, one pass, FP32 accumulate */
 #define CC_TIER_TF32X3 2 /* tcgen05 tf32, hi/lo split, 3 products */
 #define CC_TIER_BF16X3 3 /* tcgen05 kind::f16 bf16, hi/lo split, 3 products */

@@ -374,8 +374,8 @@ bool Engine::run(cplx alpha, const TRef &A, const TRef &B, cplx beta, const TRef
   if (ndim.empty()) ldb = 0;
 
   // small or skinny products stay on the CUDA-core path (GEMV or a few
-  // tiles); FP64 products large enough for it run on the tensor cores, exact
-  // to FP64
+  // tiles); FP64 products large enough for it run on the tensor cores, every
+  // element as accurate as an FP64 sum of its terms
   if (simt) {
     GemmDesc g;
     g.M = M; g.N = N; g.K = K;
@@ -523,14 +523,21 @@ bool Engine::run_slices(const GemmDesc &g, bool a_rows, bool b_rows) {
     const size_t per = slice_bytes(a_side, 1024, kb) / 1024 + 1;
     return static_cast<long>(cap / per) / 256 * 256;
   };
-  // (4.1 M rows: the guarded FP64 launch's grid)
-  const long mb = std::min<long>(rows_in(true, cap_a, g.M), 4000000);
+  const long mb = rows_in(true, cap_a, g.M);
   const long nb = rows_in(false, cap_b, g.N);
   if (mb < std::min<long>(g.M, 256) || nb < std::min<long>(g.N, 256)) return false;
-  void *ma, *mbuf;
+  // what the largest of the blocks below needs (the last ones may be split
+  // further along K than the others)
+  size_t sb = 0;
+  for (const long K : {std::min(kb, g.K), (g.K - 1) % kb + 1})
+    for (const long M : {std::min(mb, g.M), (g.M - 1) % mb + 1})
+      for (const long N : {std::min(nb, g.N), (g.N - 1) % nb + 1})
+        sb = std::max(sb, slice_scratch_bytes(M, N, K, num_sms));
+  void *ma, *mbuf, *scratch;
   try {
     ma = plane(SLICE_SLOT_A, slice_bytes(true, mb, kb));
     mbuf = plane(SLICE_SLOT_B, slice_bytes(false, nb, kb));
+    scratch = plane(SLICE_SLOT_S, sb);
   } catch (const Error &e) {
     if (e.code != CC_ERR_OOM) throw;
     ++gen;  // a plane may have been given up
@@ -569,7 +576,7 @@ bool Engine::run_slices(const GemmDesc &g, bool a_rows, bool b_rows) {
         oa.rows_unit = a_rows;
         {
           Region r = region("slice pack");
-          slice_pack(&oa, &s.A, m0 == 0 ? &ob : nullptr, &s.B, K, st, num_sms);
+          slice_pack(&oa, &s.A, m0 == 0 ? &ob : nullptr, &s.B, K, scratch, st, num_sms);
         }
         s.cm = g.cm;
         s.cn = g.cn;
@@ -585,6 +592,10 @@ bool Engine::run_slices(const GemmDesc &g, bool a_rows, bool b_rows) {
         s.src.B = ob.src;
         s.src.bn = ob.rt;
         s.src.bk = ob.kt;
+        s.a_rows = a_rows;
+        s.b_rows = b_rows;
+        s.scratch = scratch;
+        s.scratch_bytes = sb;
         Region r = region("slice gemm");
         gemm_slices(s, st, err_flag, num_sms);
       }

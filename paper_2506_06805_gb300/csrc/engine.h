@@ -109,7 +109,7 @@ class Engine {
   // and SLICE_BUDGET
   size_t slice_budget(int which, size_t need);
   static constexpr size_t SLICE_BUDGET = size_t(4) << 30;
-  static constexpr int SLICE_SLOT_A = 1000, SLICE_SLOT_B = 1001;
+  static constexpr int SLICE_SLOT_A = 1000, SLICE_SLOT_B = 1001, SLICE_SLOT_S = 1002;
   void clear_cache() {
     cache_.clear();
     packs_.clear();

@@ -1,4 +1,5 @@
-// Complex FP64 GEMM on the FP64 pipe (FP64 products too small for digit planes).
+// Complex FP64 GEMM on the FP64 pipe (FP64 products too small for digit planes,
+// and those without room for them).
 //
 // C(m, n) = alpha * sum_k A(m, k) B(n, k) + beta * C(m, n) with operands
 // gathered through offset tables (see GemmDesc). 64 x 64 complex output tile
@@ -21,9 +22,7 @@ __global__ void __launch_bounds__(256)
                  const long *__restrict__ ak, long lda, bool conjA, const double2 *__restrict__ B,
                  const long *__restrict__ bn, const long *__restrict__ bk, long ldb, bool conjB,
                  double2 *C, const long *__restrict__ cm, const long *__restrict__ cn, long ldc,
-                 double2 alpha, double2 beta, long k_per_split, bool atomic,
-                 const int *__restrict__ flag_a, const int *__restrict__ flag_b) {
-  if (flag_a && (*flag_a | *flag_b) == 0) return;  // guarded launch (gemm_f64_if)
+                 double2 alpha, double2 beta, long k_per_split, bool atomic) {
   __shared__ double2 As[TK][TM + 1];
   __shared__ double2 Bs[TK][TN + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -535,17 +534,7 @@ void gemm_f64(const GemmDesc &g, cudaStream_t st, int num_sms) {
   if (grid.y > 65535) fail(CC_ERR_ARG, "gemm_f64: M too large");
   zgemm_kernel<<<grid, 256, 0, st>>>(g.M, g.N, g.K, g.A, g.am, g.ak, g.lda, g.conjA, g.B, g.bn, g.bk,
                                      g.ldb, g.conjB, g.C, g.cm, g.cn, g.ldc, g.alpha, g.beta, kps,
-                                     atomic, nullptr, nullptr);
-  LAUNCH_CHECK();
-  count_launch();
-}
-
-void gemm_f64_if(const GemmDesc &g, const int *flag_a, const int *flag_b, cudaStream_t st) {
-  dim3 grid(static_cast<unsigned>((g.N + TN - 1) / TN), static_cast<unsigned>((g.M + TM - 1) / TM), 1);
-  if (grid.y > 65535) fail(CC_ERR_ARG, "gemm_f64_if: M too large");
-  zgemm_kernel<<<grid, 256, 0, st>>>(g.M, g.N, g.K, g.A, g.am, g.ak, g.lda, g.conjA, g.B, g.bn, g.bk,
-                                     g.ldb, g.conjB, g.C, g.cm, g.cn, g.ldc, g.alpha, g.beta, g.K,
-                                     false, flag_a, flag_b);
+                                     atomic);
   LAUNCH_CHECK();
   count_launch();
 }

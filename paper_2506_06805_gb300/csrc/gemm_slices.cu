@@ -8,8 +8,9 @@
 // Algorithms 59, 95 (2012), and Mukunoki et al., ISC 2020, for FP16 tensor
 // cores). The product is
 //   sum_g 2^(-9 (g - 1)) D_g,  D_g = sum_{i + j = g + 1} d_i(A) d_j(B)^T,
-// for g = 1 .. 7: 28 digit products; what is left out is below 2^-63 of the
-// two rows' largest magnitudes per term. Each digit product is at most 2^16
+// for g = 1 .. 7: 28 digit products. What is left out (groups 8 .. 13, the
+// rounding to 63 bits) is at most 2^-60 2^(Ea + Eb) per real term, 2^-62.9
+// sqrt(K) 2^(Ea + Eb) RMS over K complex ones. Each digit product is at most 2^16
 // in magnitude, so 256 of them (four K blocks of 64) add up without any
 // rounding in the FP32 accumulators of tcgen05.mma; the epilogue warps then
 // move the sums out of TMEM: groups 7 and 6 into FP32 (whose rounding lies
@@ -27,9 +28,20 @@
 // 0.57 ms, ladder at o = 15, v = 131, X = 517 983 -> 21 ms, FP64 residual at
 // o = 12, v = 72, X = 288 80.7 -> 5.1 ms.
 //
-// Rows that hold an Inf or NaN cannot be cut: the packing raises a flag on
-// the device, the slice kernel then stores nothing, and a guarded launch of
-// the FP64 kernel, which otherwise returns at once, computes the product.
+// That error is relative to the rows' largest magnitudes, FP64's (2^-55 to 2^-54
+// RMS) to S = sum_k |a_mk| |b_nk|, which is far smaller where large elements of
+// A meet small ones of B (columns scaled one way in A and the other in B,
+// sparse rows, small imaginary parts). So an eighth plane holds the rounded
+// magnitudes, whose product, one more beside the 28, gives S of every real and
+// imaginary part, and elements with 0 < S < 2^-7 sqrt(K) 2^(Ea + Eb) are not
+// stored but listed for slice_fix_kernel (where group 5 is in FP32, whose error
+// grows by another 2^-63.8 K 2^(Ea + Eb), those below the larger of 2^-4 sqrt(K)
+// and 2^-8 K), which computes them on the FP64 pipe. So are the elements
+// of rows with an Inf or NaN, which cannot be cut. RMS error over S in units of
+// 2^-53 (1536 x 1000 x 1200, here / FP64 kernel): normal operands 0.024 / 0.47,
+// columns scaled by 10^(+-2 k / K) 0.045 / 0.47, by 10^(+-3 k / K) and more
+// (every element listed) 0.071 / 0.47, where it takes 15.3 ms against 14.7 on
+// the FP64 pipe alone and 0.59 with none listed.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -42,7 +54,8 @@ namespace cdfns {
 
 namespace {
 
-constexpr int NS = SLICE_COUNT;  // digits per element
+constexpr int NS = SLICE_COUNT;  // digits per element; plane NS holds the magnitudes
+constexpr int PATCH_M = 16, PATCH_N = 32;  // complex elements of one epilogue warp
 constexpr int SBN = 128;         // output columns per tile
 constexpr int SKB = 2;           // K blocks of 64 per shared-memory slot and step
 constexpr int CHUNK = 2;         // steps per TMEM accumulation (at most 256 terms)
@@ -59,14 +72,57 @@ constexpr int SLICE_THREADS = (EPI_WARPS + 4) * 32;
 
 enum { SW_STORE = 0, SW_ADD = 1, SW_BETA = 2 };
 
+// Elements that the digits are not accurate enough for, per K split: those of
+// patches with few of them by themselves, from the front of the list, entry
+// patch << 16 | element; other patches in units of FIX_UNIT elements, from its
+// back, entry patch << 16 | unit, and as a mask with one bit per column.
+constexpr int FIX_THREADS = 256, FIX_K = 32, FIX_CHUNK = 512;
+constexpr int FIX_BLOCKS = 3;          // per SM
+// (units of 64 read their operands more often, 16.9 ms against 15.3 where a
+// product of 1536 x 1000 x 1200 is all units; 256 take 8 us longer where few
+// SMs have one)
+constexpr int FIX_UNIT = 128;
+constexpr int FIX_FEW = 8;
+struct FixList {
+  int *queue;                // elements, units, next unit
+  unsigned *mask;            // [patch][PATCH_M]
+  unsigned long long *list;  // [patches * FIX_FEW]
+  long patches;              // along m, n and the K splits
+};
+
+// a warp's entries: left = the bits of complex row lane / 2 of patch pt
+__device__ __noinline__ void fix_push(const FixList &x, long pt, unsigned left) {
+  const int lane = threadIdx.x & 31;
+  const unsigned w = lane & 1 ? 0u : left;
+  const int n = __reduce_add_sync(0xffffffffu, __popc(w));
+  const unsigned long long id = static_cast<unsigned long long>(pt) << 16;
+  if (n > FIX_FEW) {
+    if ((lane & 1) == 0) x.mask[pt * PATCH_M + (lane >> 1)] = left;
+    const int units = (n + FIX_UNIT - 1) / FIX_UNIT;
+    if (lane == 0) {
+      const int at = atomicAdd(&x.queue[1], units);
+      for (int u = 0; u < units; ++u) x.list[x.patches * FIX_FEW - 1 - at - u] = id | u;
+    }
+    return;
+  }
+  int at = 0;
+  if (lane == 0) at = atomicAdd(&x.queue[0], n);
+  at = __shfl_sync(0xffffffffu, at, 0);
+  for (int l = 0; l < 32; l += 2) {
+    const int c = __popc(__shfl_sync(0xffffffffu, w, l));
+    if (l < lane) at += c;
+  }
+  for (unsigned b = w; b; b &= b - 1) x.list[at++] = id | ((lane >> 1) * PATCH_N + __ffs(b) - 1);
+}
+
 struct alignas(64) SliceArgs {
   CUtensorMap mA, mB;  // [slice][row][Kp] planes as one matrix of slice * rows rows
   long M, N;           // complex rows, columns of this product
   long rows_a, rows_b; // plane rows per slice
   long a_row0, b_row0; // first plane row of this product
   const int *ea, *eb;  // per complex row: biased exponent of the largest magnitude
-  const int *fa, *fb;  // != 0: the operand holds Inf or NaN
   const float *na, *nb;  // per complex row: squared 2-norm over 4^E
+  FixList fix;           // elements left to slice_fix_kernel
   double2 *C;
   const long *cm, *cn;
   long ldc;
@@ -185,6 +241,7 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
   constexpr int UNIT_ROWS = PAIR ? 2 * BM : BM;
   constexpr uint32_t IDESC = make_idesc(UNIT_ROWS, SBN, 0u);
   constexpr int COLS = SBN * 4 / EPI_WARPS;  // columns per epilogue warp
+  static_assert(COLS == PATCH_N, "one mask bit per column");
   constexpr uint32_t TMEM_COLS = 512;
 
   extern __shared__ uint8_t smem_raw[];
@@ -250,11 +307,13 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
           const int kb1 = min(P.num_kb, kb0 + P.kb_per_split);
           const int y = is_a ? static_cast<int>(P.a_row0) + m_tile * UNIT_ROWS + TC_RANK * BM
                              : static_cast<int>(P.b_row0) + n_tile * SBN + (PAIR ? TC_RANK * (SBN / 2) : 0);
-          for (int G = NS; G >= 1 && ok; G -= 2)
+          // (the magnitudes first, plane NS of both; then the digits)
+          for (int G = NS + 2; G >= 1 && ok; G -= 2)
             for (int kb = kb0; kb < kb1 && ok; kb += SKB) {
               const int nb = min(SKB, kb1 - kb);
-              int yi = is_a ? y : y + (G - 1) * rows;  // A's digits ascend, B's descend
-              for (int i = 0; i < G; ++i, yi += is_a ? rows : -rows) {
+              const bool mag = G > NS;
+              int yi = mag ? y + NS * rows : is_a ? y : y + (G - 1) * rows;  // A's digits ascend, B's descend
+              for (int i = 0; i < (mag ? 1 : G); ++i, yi += is_a ? rows : -rows) {
                 if (!mbar_wait(&empty[s], par, P.wait_ns)) {
                   atomicExch(P.err, 1);
                   ok = false;
@@ -343,6 +402,13 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
           slice_coords(P, t, m_tile, n_tile, z);
           const int kb0 = z * P.kb_per_split;
           const int nkb = min(P.num_kb, kb0 + P.kb_per_split) - kb0;
+          int cntm = 0, bufm = 0;  // the magnitudes' product: one accumulation
+          for (int kb = 0; kb < nkb && ok; kb += SKB) {
+            if (!(ok = next_a() && next_b() && product(min(SKB, nkb - kb), cntm, bufm))) break;
+            mma_commit_both<PAIR>(&emptyB[sb]);
+            mma_commit_both<PAIR>(&emptyA[sa]);
+          }
+          if (ok) hand_over(cntm, bufm);
           for (int G = NS; G >= 1 && ok; G -= 2) {
             int cnt0 = 0, cnt1 = 0, buf0 = 0, buf1 = 0;  // groups G and G - 1
             for (int kb = 0; kb < nkb && ok; kb += SKB) {
@@ -467,6 +533,34 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
         u = max(0, (e - 18) / 2);
         if (u == 5) u = 6;
       }
+      // Elements whose S = sum_k |a||b| (the magnitudes' product, over 2^(Ea +
+      // Eb - 30)) is too small against the rows' largest magnitudes for the
+      // digits to be as accurate as FP64, and those of rows or columns with an
+      // Inf or NaN (exponent field 2047): one bit per column in this lane's
+      // mask, left to slice_fix_kernel. S = 0 has no nonzero term: 0 exactly.
+      unsigned left;
+      {
+        const float rk = sqrtf(32.0f * static_cast<float>(nkb));
+        const float thr = 0x1p30f * rk * (u ? fmaxf(0x1p-4f, 0x1p-8f * rk) : 0x1p-7f);
+        left = 0;
+        const int buf = bq.pop();
+        drain(buf, [&](int j, const float (&x)[16]) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) left |= (x[k] > 0.f && x[k] < thr) ? 1u << (j + k) : 0u;
+        });
+        bq.push(buf);
+        if (!ok) break;
+        const bool col = nbase + lane < P.N;
+        const unsigned cols = __ballot_sync(0xffffffffu, col);
+        left |= __ballot_sync(0xffffffffu, col && P.eb[P.b_row0 + nbase + lane] == 2047);
+        if (mrow >= P.M) left = 0;
+        else if (P.ea[P.a_row0 / 2 + mrow] == 2047) left = ~0u;
+        left &= cols;
+        left |= __shfl_xor_sync(0xffffffffu, left, 1);
+        const long pt = (static_cast<long>(z) * P.m_tiles * (UNIT_ROWS / 2 / PATCH_M) + mbase / PATCH_M) *
+                            P.n_tiles * (SBN / PATCH_N) + nbase / PATCH_N;
+        if (__any_sync(0xffffffffu, left != 0)) fix_push(P.fix, pt, left);
+      }
       {
         float lf[COLS];
 #pragma unroll
@@ -538,7 +632,6 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
       // eight, column) of complex results on the way out. The conversion
       // sits on the way out, in a loop: unrolled over the accumulators it was
       // far larger than the instruction cache (110 000 clocks a tile).
-      const bool skip = (*P.fa | *P.fb) != 0;
       const int ea = (mrow < P.M ? P.ea[P.a_row0 / 2 + mrow] : 1) - 2 * 1022 - 61 + (P.alpha_p2 ? P.alpha_e : 0);
       const int ebl = nbase + lane < P.N ? P.eb[P.b_row0 + nbase + lane] : 1;
       long roff = 0;
@@ -563,13 +656,14 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
         const int c = 4 * seg + col;
         const int eb = __shfl_sync(0xffffffffu, ebl, c);
         const long n = nbase + c;
-        const bool col_ok = n < P.N && !skip;
+        const bool col_ok = n < P.N;
         const long cno = col_ok ? (P.cn ? P.cn[n] : n) : 0;
 #pragma unroll 1
         for (int rr = 0; rr < 2; ++rr) {
           const int r = 8 * rr + hf;
           const long ro = __shfl_sync(0xffffffffu, roff, r);
           const int e = __shfl_sync(0xffffffffu, ea, 2 * r) + eb;
+          const unsigned skip = __shfl_sync(0xffffffffu, left, 2 * r);
           double v[2];
 #pragma unroll
           for (int w = 0; w < 2; ++w) {
@@ -580,7 +674,7 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
             v[w] = scale_exp(d, e);
             if (P.alpha_neg) v[w] = __hiloint2double(__double2hiint(v[w]) ^ 0x80000000, __double2loint(v[w]));
           }
-          if (!col_ok || mbase + r >= P.M) continue;
+          if (!col_ok || mbase + r >= P.M || ((skip >> c) & 1u)) continue;
           double2 *o = P.C + ro + cno;
           double2 y = make_double2(v[0], v[1]);
           if (!P.alpha_p2) y = cmul(P.alpha, y);
@@ -628,20 +722,21 @@ struct SideArgs {
   long ld, rows;
   bool conj, rows_unit, expand;
   __half *planes;
-  int *e;     // [rows] exponent fields, then the Inf/NaN flag
+  int *e;     // [rows] exponent fields
   float *n2;  // [rows] squared 2-norms over 4^E
 };
 
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
-// e[row] = the largest exponent field of the row's components (at least 1),
-// e[rows] != 0 if any is 2047. One warp per item: 32 rows x 16 k with lanes
+// e[row] = the largest exponent field of the row's components (at least 1;
+// 2047: an Inf or NaN). One warp per item: 32 rows x 16 k with lanes
 // along the rows where those are neighbours in memory, else one row x 256 k
 // with lanes along k, 8 loads in flight: on small operands the time is one
 // item's latency (items four times as long took 36 us at any size), on
 // large ones the read of the operand.
 __global__ void __launch_bounds__(256) slice_exp_kernel(SideArgs a, SideArgs b, long K, long items_a,
-                                                        long items) {
+                                                        long items, int *reset) {
+  if (reset && blockIdx.x == 0 && threadIdx.x < SLICE_RESET_BYTES / sizeof(int)) reset[threadIdx.x] = 0;
   const int lane = threadIdx.x & 31;
   const long nw = static_cast<long>(gridDim.x) * 8;
   for (long w = blockIdx.x * 8L + (threadIdx.x >> 5); w < items; w += nw) {
@@ -659,7 +754,6 @@ __global__ void __launch_bounds__(256) slice_exp_kernel(SideArgs a, SideArgs b, 
           m = max(m, max(exp_field(x.x), exp_field(x.y)));
         }
         atomicMax(&s.e[r], m);
-        if (m == 2047) s.e[s.rows] = 1;
       }
     } else {
       const long nk = (K + 255) / 256;
@@ -671,10 +765,7 @@ __global__ void __launch_bounds__(256) slice_exp_kernel(SideArgs a, SideArgs b, 
         m = max(m, max(exp_field(x.x), exp_field(x.y)));
       }
       m = __reduce_max_sync(0xffffffffu, m);
-      if (lane == 0) {
-        atomicMax(&s.e[r], m);
-        if (m == 2047) s.e[s.rows] = 1;
-      }
+      if (lane == 0) atomicMax(&s.e[r], m);
     }
   }
 }
@@ -699,10 +790,11 @@ __device__ __forceinline__ __half2 digits2(int x, int y) {
   return __hsub2(*reinterpret_cast<const __half2 *>(&u), __float2half2_rn(1280.0f));
 }
 
-// one complex element's digits into its place of every slice; the lanes of a
-// warp hold 32 neighbouring k of one row
+// one complex element's digits and magnitudes into its place of every plane;
+// the lanes of a warp hold 32 neighbouring k of one row
 __device__ __forceinline__ void store_digits(const SideArgs &s, long r, long kc, long Kp, double2 x,
                                              int field) {
+  const bool nr = (__double_as_longlong(x.x) << 1) != 0, ni = (__double_as_longlong(x.y) << 1) != 0;
   long long re = to_fixed(x.x, field), im = to_fixed(x.y, field);
   if (s.conj) im = -im;
   // |x|^2 4^-E of this element, summed over the warp's 32 k
@@ -714,6 +806,14 @@ __device__ __forceinline__ void store_digits(const SideArgs &s, long r, long kc,
   __half2 *pl = reinterpret_cast<__half2 *>(s.planes);
   const long hk = Kp / 2;
   const long prow = s.expand ? 2 * r : r, prows = s.expand ? 2 * s.rows : s.rows;
+  {
+    // magnitudes over 2^(E - 15); nonzero ones stay normal halves (2^-14)
+    const __half2 mg = __floats2half2_rn(fmaxf(fabsf(fr) * 32768.f, nr ? 0x1p-14f : 0.f),
+                                         fmaxf(fabsf(fi) * 32768.f, ni ? 0x1p-14f : 0.f));
+    const long o = (NS * prows + prow) * hk + kc;
+    pl[o] = mg;
+    if (s.expand) pl[o + hk] = __lowhigh2highlow(mg);
+  }
 #pragma unroll
   for (int d = NS - 1; d >= 0; --d) {
     int dr, di;
@@ -738,7 +838,7 @@ __device__ __forceinline__ void store_digits(const SideArgs &s, long r, long kc,
 
 // Digit planes of both operands: 32 x 32 tiles, read along the direction that
 // is contiguous in the source (transposed through shared memory when that is
-// the rows) and written along k. HBM bound: 16 B read, 28 B (56 B for the
+// the rows) and written along k. HBM bound: 16 B read, 32 B (64 B for the
 // expanded A side) written per element.
 __global__ void __launch_bounds__(256) slice_pack_kernel(SideArgs a, SideArgs b, long K, long Kp,
                                                          long items_a, long items) {
@@ -781,6 +881,213 @@ __global__ void __launch_bounds__(256) slice_pack_kernel(SideArgs a, SideArgs b,
   }
 }
 
+// ---------------------------------------------------------------------------
+// elements the digits are not accurate enough for, on the FP64 pipe
+// ---------------------------------------------------------------------------
+struct FixSide {
+  const double2 *p;
+  const long *rt, *kt;
+  long ld;
+  bool conj, rows_unit;
+};
+struct FixArgs {
+  long M, N, K, k_per_split;
+  long pm, pn;  // patches along m and along n
+  FixList fix;
+  const int *err;
+  FixSide A, B;
+  double2 *C;
+  const long *cm, *cn;
+  long ldc;
+  double2 alpha, beta;
+  int wmode;
+};
+// ROWS rows x FIX_K of an operand on their way into shared memory [k][row],
+// read along whichever of the two is contiguous. Rows and k beyond the end
+// read the last valid ones, so that a thread's loads are in flight together
+// (tested one by one they ran one after another, 9 us a tile); k beyond the
+// end count as zero, rows beyond it are not used.
+template <int ROWS>
+struct FixTile {
+  static constexpr int N = ROWS * FIX_K / FIX_THREADS;
+  long ro[N];
+  double2 x[N];
+  __device__ __forceinline__ int row(const FixSide &s, int i) const {
+    const int t = threadIdx.x + FIX_THREADS * i;
+    return s.rows_unit ? t % ROWS : t / FIX_K;
+  }
+  __device__ __forceinline__ int col(const FixSide &s, int i) const {
+    const int t = threadIdx.x + FIX_THREADS * i;
+    return s.rows_unit ? t / ROWS : t % FIX_K;
+  }
+  __device__ __forceinline__ void rows(const FixSide &s, long r0, long rows) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const long r = min(r0 + row(s, i), rows - 1);
+      ro[i] = s.rt ? s.rt[r] : r * s.ld;
+    }
+  }
+  __device__ __forceinline__ void load(const FixSide &s, long k0, long k1) {
+    long ko[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const long k = min(k0 + col(s, i), k1 - 1);
+      ko[i] = s.kt ? s.kt[k] : k;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = s.p[ro[i] + ko[i]];
+  }
+  __device__ __forceinline__ void store(const FixSide &s, long k0, long k1, double2 (&to)[FIX_K][ROWS + 1]) const {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int c = col(s, i);
+      double2 y = x[i];
+      if (s.conj) y.y = -y.y;
+      to[c][row(s, i)] = k0 + c < k1 ? y : make_double2(0.0, 0.0);
+    }
+  }
+};
+
+struct FixPatch {
+  long z, m0, n0, k0, k1;  // split, first row and column, K range
+  unsigned cols;           // columns within the product
+};
+__device__ __forceinline__ FixPatch fix_patch(const FixArgs &P, long pt) {
+  FixPatch q;
+  q.z = pt / (P.pm * P.pn);
+  const long mn = pt - q.z * (P.pm * P.pn);
+  q.m0 = mn / P.pn * PATCH_M;
+  q.n0 = mn % P.pn * PATCH_N;
+  q.k0 = q.z * P.k_per_split;
+  q.k1 = min(P.K, q.k0 + P.k_per_split);
+  q.cols = q.n0 + PATCH_N <= P.N ? ~0u : q.n0 < P.N ? (1u << (P.N - q.n0)) - 1u : 0u;
+  return q;
+}
+__device__ __forceinline__ unsigned fix_mask(const FixArgs &P, const FixPatch &q, long pt, int r) {
+  return q.m0 + r < P.M ? P.fix.mask[pt * PATCH_M + r] & q.cols : 0u;
+}
+
+__device__ __forceinline__ void fix_store(const FixArgs &P, long m, long n, double2 x) {
+  double2 *o = P.C + (P.cm ? P.cm[m] : m * P.ldc) + (P.cn ? P.cn[n] : n);
+  const double2 y = cmul(P.alpha, x);
+  if (P.wmode == SW_ADD) {
+    atomicAdd(&o->x, y.x);
+    atomicAdd(&o->y, y.y);
+  } else {
+    *o = P.wmode == SW_STORE ? y : cadd(y, cmul(P.beta, *o));
+  }
+}
+
+// one element by a warp, the lanes striding k
+__device__ __forceinline__ void fix_element(const FixArgs &P, const FixPatch &q, int r, int c) {
+  const long m = q.m0 + r, n = q.n0 + c;
+  const double2 *pa = P.A.p + (P.A.rt ? P.A.rt[m] : m * P.A.ld);
+  const double2 *pb = P.B.p + (P.B.rt ? P.B.rt[n] : n * P.B.ld);
+  double2 s = make_double2(0.0, 0.0);
+  for (long k = q.k0 + (threadIdx.x & 31); k < q.k1; k += 128) {
+    double2 a[4], b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const long kk = min(k + 32 * u, q.k1 - 1);
+      a[u] = pa[P.A.kt ? P.A.kt[kk] : kk];
+      b[u] = pb[P.B.kt ? P.B.kt[kk] : kk];
+    }
+    double2 x = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (P.A.conj) a[u].y = -a[u].y;
+      if (P.B.conj) b[u].y = -b[u].y;
+      if (k + 32 * u < q.k1) x = cfma(a[u], b[u], x);
+    }
+    s = cadd(s, x);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+  }
+  if ((threadIdx.x & 31) == 0) fix_store(P, m, n, s);
+}
+
+// The elements slice_gemm_kernel has listed, over the K range of their split.
+// Single ones (the usual case: near zeros of structured operands): a warp
+// each. A unit of a patch with more: a block, its operands through shared
+// memory; blocks draw the units from a queue. Sums run over 8 terms and over
+// 512 / 8 such runs at a time, as short as those of the FP64 kernels' warps.
+__global__ void __launch_bounds__(FIX_THREADS, FIX_BLOCKS) slice_fix_kernel(const FixArgs P) {
+  __shared__ double2 As[FIX_K][PATCH_M + 1], Bs[FIX_K][PATCH_N + 1];
+  __shared__ unsigned short el[FIX_UNIT];
+  __shared__ int unit;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int n_el = P.fix.queue[0], n_units = P.fix.queue[1];
+  if (*P.err) return;  // a wait has expired
+  for (long f = blockIdx.x * (FIX_THREADS / 32L) + warp; f < n_el; f += gridDim.x * (FIX_THREADS / 32L)) {
+    const unsigned long long e = P.fix.list[f];
+    const int c = e & 0xffffu;
+    fix_element(P, fix_patch(P, static_cast<long>(e >> 16)), c / PATCH_N, c % PATCH_N);
+  }
+  if (n_units) {
+    for (;;) {
+      if (t == 0) unit = atomicAdd(&P.fix.queue[2], 1);
+      __syncthreads();
+      if (unit >= n_units) break;
+      const unsigned long long id = P.fix.list[P.fix.patches * FIX_FEW - 1 - unit];
+      const long pt = static_cast<long>(id >> 16);
+      const FixPatch q = fix_patch(P, pt);
+      const int first = static_cast<int>(id & 0xffffu) * FIX_UNIT;
+      int n = 0;
+      for (int r = 0; r < PATCH_M; ++r) {
+        const unsigned w = fix_mask(P, q, pt, r);
+        const int at = n + __popc(w & ((1u << lane) - 1u)) - first;
+        if (warp == 0 && ((w >> lane) & 1u) && at >= 0 && at < FIX_UNIT)
+          el[at] = static_cast<unsigned short>(r * PATCH_N + lane);
+        n += __popc(w);
+      }
+      __syncthreads();
+      // two or four threads an element, each every second or fourth k
+      const int m = min(n - first, FIX_UNIT), sl = m > FIX_THREADS / 4 ? 1 : 2, sp = 1 << sl;
+      const int sub = t & (sp - 1);
+      const bool on = (t >> sl) < m;
+      const int e = on ? el[t >> sl] : 0, r = e / PATCH_N, c = e % PATCH_N;
+      double2 s = make_double2(0.0, 0.0);
+      FixTile<PATCH_M> ta;
+      FixTile<PATCH_N> tb;
+      ta.rows(P.A, q.m0, P.M);
+      tb.rows(P.B, q.n0, P.N);
+      for (long kc = q.k0; kc < q.k1; kc += FIX_CHUNK) {
+        const long ke = min(q.k1, kc + FIX_CHUNK);
+        double2 y = make_double2(0.0, 0.0);
+        for (long k = kc; k < ke; k += FIX_K) {
+          ta.load(P.A, k, q.k1);
+          tb.load(P.B, k, q.k1);
+          ta.store(P.A, k, q.k1, As);
+          tb.store(P.B, k, q.k1, Bs);
+          __syncthreads();
+          if (on) {
+            const double2 *a = &As[sub][r], *b = &Bs[sub][c];
+            for (int g = 0; g < FIX_K >> sl; g += 8) {
+              double2 x = make_double2(0.0, 0.0);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                x = cfma(*a, *b, x);
+                a += sp * (PATCH_M + 1);
+                b += sp * (PATCH_N + 1);
+              }
+              y = cadd(y, x);
+            }
+          }
+          __syncthreads();
+        }
+        s = cadd(s, y);
+      }
+      for (int o = sp / 2; o > 0; o >>= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+      }
+      if (on && sub == 0) fix_store(P, q.m0 + r, q.n0 + c, s);
+    }
+  }
+}
+
 template <int STAGES, bool PAIR>  // STAGES slots of SKB K blocks for each operand
 void launch_slices(SliceArgs &a, const SlicePlanes &A, const SlicePlanes &B, int units, int sms,
                    cudaStream_t st) {
@@ -794,8 +1101,8 @@ void launch_slices(SliceArgs &a, const SlicePlanes &A, const SlicePlanes &B, int
     return true;
   }();
   (void)attr;
-  a.mA = make_map(A.planes, NS * A.plane_rows, A.Kp, BM, 2);
-  a.mB = make_map(B.planes, NS * B.plane_rows, B.Kp, PAIR ? SBN / 2 : SBN, 2);
+  a.mA = make_map(A.planes, SLICE_PLANES * A.plane_rows, A.Kp, BM, 2);
+  a.mB = make_map(B.planes, SLICE_PLANES * B.plane_rows, B.Kp, PAIR ? SBN / 2 : SBN, 2);
   if constexpr (!PAIR) {
     kern<<<static_cast<unsigned>(std::min(units, sms)), SLICE_THREADS, SMEM, st>>>(a);
   } else {
@@ -824,8 +1131,8 @@ void launch_slices(SliceArgs &a, const SlicePlanes &A, const SlicePlanes &B, int
   count_launch();
 }
 
-// Work of one launch in tile-K-blocks per resident unit (28 digit products of
-// a K block), the epilogue counted as 3 K blocks: what a split is chosen by.
+// Work of one launch in tile-K-blocks per resident unit (29 products of a K
+// block), the epilogue counted as 3 K blocks: what a split is chosen by.
 double makespan(long tiles, long nkb, long split, long P) {
   const long per = (nkb + split - 1) / split;
   return static_cast<double>((tiles * ((nkb + per - 1) / per) + P - 1) / P) * (static_cast<double>(per) + 3.0);
@@ -852,18 +1159,18 @@ SideArgs side(const SliceOperand &x, const SlicePlanes &p, bool expand) {
 long slice_kp(long K) { return (2 * K + 63) / 64 * 64; }
 
 namespace {
-// [exponents, flag, norms, padded to 256 B][NS planes]
-size_t slice_head(long rows) { return (sizeof(int) * (2 * rows + 1) + 255) / 256 * 256; }
+// [exponents, norms, padded to 256 B][planes]
+size_t slice_head(long rows) { return (sizeof(int) * 2 * rows + 255) / 256 * 256; }
 }  // namespace
 
 size_t slice_bytes(bool a_side, long rows, long K) {
-  return slice_head(rows) + sizeof(__half) * NS * (a_side ? 2 : 1) * rows * slice_kp(K);
+  return slice_head(rows) + sizeof(__half) * SLICE_PLANES * (a_side ? 2 : 1) * rows * slice_kp(K);
 }
 
 SlicePlanes slice_planes(void *mem, bool a_side, long rows, long K) {
   SlicePlanes p;
   p.e = static_cast<int *>(mem);
-  p.n2 = reinterpret_cast<float *>(p.e + rows + 1);
+  p.n2 = reinterpret_cast<float *>(p.e + rows);
   p.planes = static_cast<char *>(mem) + slice_head(rows);
   p.rows = rows;
   p.plane_rows = (a_side ? 2 : 1) * rows;
@@ -872,7 +1179,7 @@ SlicePlanes slice_planes(void *mem, bool a_side, long rows, long K) {
 }
 
 void slice_pack(const SliceOperand *A, const SlicePlanes *pa, const SliceOperand *B,
-                const SlicePlanes *pb, long K, cudaStream_t st, int num_sms) {
+                const SlicePlanes *pb, long K, void *scratch, cudaStream_t st, int num_sms) {
   SideArgs a = {}, b = {};
   long exp_a = 0, exp_b = 0, tiles_a = 0, tiles_b = 0, Kp = 0;
   auto setup = [&](const SliceOperand &x, const SlicePlanes &p, bool expand, SideArgs &s, long &ne,
@@ -881,14 +1188,14 @@ void slice_pack(const SliceOperand *A, const SlicePlanes *pa, const SliceOperand
     ne = x.rows_unit ? (x.rows + 31) / 32 * ((K + 15) / 16) : x.rows * ((K + 255) / 256);
     nt = (x.rows + 31) / 32 * (p.Kp / 64);
     Kp = p.Kp;
-    CUDA_CHECK(cudaMemsetAsync(p.e, 0, sizeof(int) * (2 * x.rows + 1), st));
+    CUDA_CHECK(cudaMemsetAsync(p.e, 0, sizeof(int) * 2 * x.rows, st));
   };
   if (A) setup(*A, *pa, true, a, exp_a, tiles_a);
   if (B) setup(*B, *pb, false, b, exp_b, tiles_b);
   const long ne = exp_a + exp_b, nt = tiles_a + tiles_b;
   if (nt == 0) return;
   slice_exp_kernel<<<static_cast<unsigned>(std::min<long>((ne + 7) / 8, 8L * num_sms)), 256, 0, st>>>(
-      a, b, K, exp_a, ne);
+      a, b, K, exp_a, ne, static_cast<int *>(scratch));
   LAUNCH_CHECK();
   slice_pack_kernel<<<static_cast<unsigned>(std::min<long>(nt, 32L * num_sms)), 256, 0, st>>>(
       a, b, K, Kp, tiles_a, nt);
@@ -896,10 +1203,60 @@ void slice_pack(const SliceOperand *A, const SlicePlanes *pa, const SliceOperand
   count_launch(2);
 }
 
+namespace {
+// Tiles and K split of an M x N product over num_kb blocks of 64
+struct SlicePlan {
+  bool pair;
+  int kb_per_split, k_splits, m_tiles, n_tiles;
+  long units() const { return static_cast<long>(m_tiles) * n_tiles * k_splits; }
+  long patches_m() const { return static_cast<long>(m_tiles) * ((pair ? BM : BM / 2) / PATCH_M); }
+  long patches_n() const { return static_cast<long>(n_tiles) * (SBN / PATCH_N); }
+  long patches() const { return patches_m() * patches_n() * k_splits; }
+};
+
+SlicePlan slice_plan(long M, long N, long num_kb, int num_sms) {
+  // CTA pairs when they leave no more work to the slowest SM than single CTAs
+  // (whose 128-row tiles pad less but stream a third more per product)
+  const long nt = (N + SBN - 1) / SBN;
+  const long t1 = (2 * M + BM - 1) / BM * nt, t2 = (2 * M + 2 * BM - 1) / (2 * BM) * nt;
+  auto best_split = [&](long tiles, long P, double &cost) {
+    long sp = 1;
+    cost = makespan(tiles, num_kb, 1, P);
+    if (tiles < 2 * P)
+      for (long s = 2; s <= std::min<long>(num_kb, 64); ++s) {
+        // a split adds its partial sums to the output in FP64: one more K
+        // block's worth of epilogue
+        const double c = makespan(tiles, num_kb, s, P) + 1.0;
+        if (c < 0.95 * cost) {
+          cost = c;
+          sp = s;
+        }
+      }
+    return sp;
+  };
+  double c1, c2;
+  const long s1 = best_split(t1, num_sms, c1), s2 = best_split(t2, num_sms / 2, c2);
+  SlicePlan p;
+  p.pair = c2 <= 1.05 * c1;
+  const long split = p.pair ? s2 : s1;
+  p.kb_per_split = static_cast<int>((num_kb + split - 1) / split);
+  p.k_splits = static_cast<int>((num_kb + p.kb_per_split - 1) / p.kb_per_split);
+  p.n_tiles = static_cast<int>(nt);
+  p.m_tiles = static_cast<int>((2 * M + (p.pair ? 2 * BM : BM) - 1) / (p.pair ? 2 * BM : BM));
+  return p;
+}
+}  // namespace
+
+size_t slice_scratch_bytes(long M, long N, long K, int num_sms) {
+  if (M <= 0 || N <= 0) return 0;
+  return SLICE_RESET_BYTES + (sizeof(unsigned) * PATCH_M + sizeof(unsigned long long) * FIX_FEW) *
+                                 slice_plan(M, N, slice_kp(K) / 64, num_sms).patches();
+}
+
 void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
   if (g.M <= 0 || g.N <= 0) return;
   const SlicePlanes &A = g.A, &B = g.B;
-  if (A.Kp != B.Kp || NS * A.plane_rows > 0x7fffffffL || NS * B.plane_rows > 0x7fffffffL)
+  if (A.Kp != B.Kp || SLICE_PLANES * A.plane_rows > 0x7fffffffL || SLICE_PLANES * B.plane_rows > 0x7fffffffL)
     fail(CC_ERR_ARG, "gemm_slices: operand planes");
   SliceArgs a = {};
   a.M = g.M;
@@ -910,8 +1267,6 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
   a.b_row0 = g.b_row0;
   a.ea = A.e;
   a.eb = B.e;
-  a.fa = A.e + A.rows;
-  a.fb = B.e + B.rows;
   a.na = A.n2;
   a.nb = B.n2;
   a.C = g.C;
@@ -929,64 +1284,58 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
   a.num_kb = static_cast<int>(A.Kp / 64);
   a.err = err;
   a.wait_ns = tc_wait_limit();
-  // CTA pairs when they leave no more work to the slowest SM than single CTAs
-  // (whose 128-row tiles pad less but stream a third more per product)
-  const long nt = (g.N + SBN - 1) / SBN;
-  const long t1 = (2 * g.M + BM - 1) / BM * nt, t2 = (2 * g.M + 2 * BM - 1) / (2 * BM) * nt;
-  auto best_split = [&](long tiles, long P, double &cost) {
-    long sp = 1;
-    cost = makespan(tiles, a.num_kb, 1, P);
-    if (tiles < 2 * P)
-      for (long s = 2; s <= std::min<long>(a.num_kb, 64); ++s) {
-        // a split adds its partial sums to the output in FP64: one more K
-        // block's worth of epilogue
-        const double c = makespan(tiles, a.num_kb, s, P) + 1.0;
-        if (c < 0.95 * cost) {
-          cost = c;
-          sp = s;
-        }
-      }
-    return sp;
-  };
-  double c1, c2;
-  const long s1 = best_split(t1, num_sms, c1), s2 = best_split(t2, num_sms / 2, c2);
-  const bool pair = c2 <= 1.05 * c1;
-  const long split = pair ? s2 : s1;
-  a.kb_per_split = static_cast<int>((a.num_kb + split - 1) / split);
-  a.k_splits = (a.num_kb + a.kb_per_split - 1) / a.kb_per_split;
-  a.n_tiles = static_cast<int>(nt);
-  a.m_tiles = static_cast<int>((2 * g.M + (pair ? 2 * BM : BM) - 1) / (pair ? 2 * BM : BM));
-  const double square = std::sqrt(static_cast<double>(pair ? num_sms / 2 : num_sms) * SBN / (pair ? 2 * BM : BM));
+  const SlicePlan p = slice_plan(g.M, g.N, a.num_kb, num_sms);
+  a.kb_per_split = p.kb_per_split;
+  a.k_splits = p.k_splits;
+  a.n_tiles = p.n_tiles;
+  a.m_tiles = p.m_tiles;
+  const double square = std::sqrt(static_cast<double>(p.pair ? num_sms / 2 : num_sms) * SBN / (p.pair ? 2 * BM : BM));
   a.group_m = std::max(1, std::min(a.m_tiles, static_cast<int>(square)));
-  const long units = static_cast<long>(a.m_tiles) * a.n_tiles * a.k_splits;
-  if (units > 0x7fffffffL) fail(CC_ERR_ARG, "gemm_slices: too many tiles");
+  if (p.units() > 0x7fffffffL) fail(CC_ERR_ARG, "gemm_slices: too many tiles");
+  if (!g.scratch || g.scratch_bytes < slice_scratch_bytes(g.M, g.N, g.src.K, num_sms) ||
+      slice_kp(g.src.K) != A.Kp)
+    fail(CC_ERR_ARG, "gemm_slices: scratch");
+  a.fix.patches = p.patches();
+  a.fix.queue = static_cast<int *>(g.scratch);
+  a.fix.list = reinterpret_cast<unsigned long long *>(static_cast<char *>(g.scratch) + SLICE_RESET_BYTES);
+  a.fix.mask = reinterpret_cast<unsigned *>(a.fix.list + p.patches() * FIX_FEW);
   a.wmode = (g.beta.x == 0.0 && g.beta.y == 0.0) ? SW_STORE
             : (g.beta.x == 1.0 && g.beta.y == 0.0) ? SW_ADD
                                                    : SW_BETA;
-  cplx guard_beta = g.beta;
   if (a.k_splits > 1) {
     scale_2d(g.C, g.cm, g.cn, g.ldc, g.M, g.N, g.beta, st);
     a.wmode = SW_ADD;
-    guard_beta = make_double2(1.0, 0.0);
   }
-  const int u = static_cast<int>(units);
-  if (pair) launch_slices<4, true>(a, A, B, u, num_sms, st);
+  const int u = static_cast<int>(p.units());
+  if (p.pair) launch_slices<4, true>(a, A, B, u, num_sms, st);
   else launch_slices<3, false>(a, A, B, u, num_sms, st);
-  // Inf or NaN in an operand: the FP64 kernel computes this product instead
-  GemmDesc f = g.src;
+  // the elements left out, on the FP64 pipe
+  FixArgs f = {};
   f.M = g.M;
   f.N = g.N;
+  f.K = g.src.K;
+  f.k_per_split = 32L * p.kb_per_split;
+  f.pm = p.patches_m();
+  f.pn = p.patches_n();
+  f.fix = a.fix;
+  f.err = err;
+  f.A = FixSide{g.src.A, g.src.am, g.src.ak, g.src.lda, g.src.conjA, g.a_rows};
+  f.B = FixSide{g.src.B, g.src.bn, g.src.bk, g.src.ldb, g.src.conjB, g.b_rows};
   f.C = g.C;
   f.cm = g.cm;
   f.cn = g.cn;
   f.ldc = g.ldc;
   f.alpha = g.alpha;
-  f.beta = guard_beta;
-  gemm_f64_if(f, a.fa, a.fb, st);
+  f.beta = g.beta;
+  f.wmode = a.wmode;
+  const long blocks = std::min<long>(f.fix.patches, static_cast<long>(FIX_BLOCKS) * num_sms);
+  slice_fix_kernel<<<static_cast<unsigned>(blocks), FIX_THREADS, 0, st>>>(f);
+  LAUNCH_CHECK();
+  count_launch();
 }
 
 // Estimated times (s) of an M x N x K product here and on the FP64 pipe. The
-// tensor side: 28 digit products of every 128 x 128 x 64 block at about 1
+// tensor side: 29 products of every 128 x 128 x 64 block at about 1
 // PF/s, an epilogue of three K blocks per tile, the planes written and read,
 // five launches. The FP64 side: 1 TF/s or its operands at 5 TB/s, on whole
 // 64 x 64 tiles where the tiled kernel takes the product (a tile's rows cost
@@ -994,8 +1343,8 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
 bool slices_pay(long M, long N, long K) {
   const double m = (2 * M + 127) / 128 * 128.0, n = (N + 127) / 128 * 128.0;
   const double kb = static_cast<double>((2 * K + 63) / 64);
-  const double mma = 2.0 * m * n * 64.0 * 28.0 * (kb + 3.0) / 1e15;
-  const double pack = (static_cast<double>(M) * K * (32 + 112) + static_cast<double>(N) * K * (32 + 56)) / 5e12;
+  const double mma = 2.0 * m * n * 64.0 * 29.0 * (kb + 3.0) / 1e15;
+  const double pack = (static_cast<double>(M) * K * (32 + 128) + static_cast<double>(N) * K * (32 + 64)) / 5e12;
   const double out = 32.0 * M * N / 5e12;
   const double t_slices = 20e-6 + std::max(mma, 20e-6) + pack + out;
   const long tm = (M + 63) / 64, tn = (N + 63) / 64;

@@ -29,14 +29,13 @@ struct GemmDesc {
 // FP64 SIMT path (CC_TIER_FP64).
 void gemm_f64(const GemmDesc &g, cudaStream_t st, int num_sms);
 
-// The plain tiled FP64 kernel of g, computed only if *flag_a or *flag_b is
-// nonzero on the device (otherwise the launch returns at once).
-void gemm_f64_if(const GemmDesc &g, const int *flag_a, const int *flag_b, cudaStream_t st);
-
 // FP64 products on the tensor cores (gemm_slices.cu): operands cut into
 // SLICE_COUNT planes of integer digits relative to each row's largest
-// magnitude, products of the planes summed exactly.
+// magnitude, products of the planes summed exactly, and a plane of magnitudes.
+// Elements that this form cannot give to FP64's accuracy are computed on the
+// FP64 pipe.
 constexpr int SLICE_COUNT = 7;
+constexpr int SLICE_PLANES = SLICE_COUNT + 1;
 struct SliceOperand {  // rows x K source elements, addressed as in GemmDesc
   const cplx *src = nullptr;
   const long *rt = nullptr, *kt = nullptr;
@@ -46,8 +45,8 @@ struct SliceOperand {  // rows x K source elements, addressed as in GemmDesc
   bool rows_unit = false;  // neighbouring rows are neighbours in memory, k is strided
 };
 struct SlicePlanes {
-  void *planes = nullptr;  // [SLICE_COUNT][plane_rows][Kp] FP16
-  int *e = nullptr;        // [rows] exponents, then the Inf/NaN flag
+  void *planes = nullptr;  // [SLICE_PLANES][plane_rows][Kp] FP16
+  int *e = nullptr;        // [rows] exponents
   float *n2 = nullptr;     // [rows] squared 2-norms relative to the row's 2^E
   long rows = 0, plane_rows = 0, Kp = 0;
 };
@@ -55,9 +54,11 @@ long slice_kp(long K);
 // bytes of an operand's planes and exponents (A side: rows expanded by two)
 size_t slice_bytes(bool a_side, long rows, long K);
 SlicePlanes slice_planes(void *mem, bool a_side, long rows, long K);  // views into slice_bytes() bytes
-// planes of one or both operands (either side may be NULL)
+// planes of one or both operands (either side may be NULL); scratch (may be
+// NULL): the first SLICE_RESET_BYTES of a product's scratch are zeroed on the way
+constexpr size_t SLICE_RESET_BYTES = 16;
 void slice_pack(const SliceOperand *A, const SlicePlanes *pa, const SliceOperand *B,
-                const SlicePlanes *pb, long K, cudaStream_t st, int num_sms);
+                const SlicePlanes *pb, long K, void *scratch, cudaStream_t st, int num_sms);
 struct SliceGemm {
   long M = 0, N = 0;             // complex rows a_row0 .. of A, rows b_row0 .. of B
   SlicePlanes A, B;
@@ -65,7 +66,15 @@ struct SliceGemm {
   cplx *C = nullptr; const long *cm = nullptr, *cn = nullptr; long ldc = 0;
   cplx alpha = {1.0, 0.0}, beta = {0.0, 0.0};
   GemmDesc src;                  // the operands themselves (A, B, K and their addressing)
+  bool a_rows = false, b_rows = false;  // their rows_unit
+  // slice_scratch_bytes() bytes, not shared with work in flight, the first
+  // SLICE_RESET_BYTES of them zero
+  void *scratch = nullptr;
+  size_t scratch_bytes = 0;
 };
+// Device bytes gemm_slices needs beside the planes (1/64 of the output, some
+// more when K is split).
+size_t slice_scratch_bytes(long M, long N, long K, int num_sms);
 void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err_flag, int num_sms);
 // whether an M x N x K FP64 product is expected to be faster this way
 bool slices_pay(long M, long N, long K);

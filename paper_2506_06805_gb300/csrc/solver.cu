@@ -612,7 +612,7 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
       pB = slice_planes(LB.p, false, vv, X);
       SliceOperand l;
       l.src = Lv; l.kt = ptab; l.ld = 1; l.rows = vv; l.rows_unit = true;
-      slice_pack(&l, &pA, &l, &pB, X, st, num_sms);
+      slice_pack(&l, &pA, &l, &pB, X, nullptr, st, num_sms);
     } else {
       LT.reset(&al, sizeof(cplx) * vv * X);
       eng.permute_into(C1(), T(Lv, "Pac", {X, v, v}), C0(), T(LT.c(), "acP", {v, v, X}));
@@ -629,7 +629,13 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
       const long np = p1 - p0;
       B(Vs, nA * per_a);
       B(W, np * n_cd);
-      for (const auto &ar : slab_rows(v, a0, nA, X)) {
+      const auto ranges = slab_rows(v, a0, nA, X);
+      size_t sb = 0;
+      if (LA.p)
+        for (const auto &ar : ranges)
+          sb = std::max(sb, slice_scratch_bytes((ar.second - ar.first) * v, (v - ar.first - 1) * v, X, num_sms));
+      void *scratch = sb ? eng.plane(Engine::SLICE_SLOT_S, sb) : nullptr;
+      for (const auto &ar : ranges) {
         const long s0 = ar.first, s1 = ar.second;
         GemmDesc g1;
         g1.M = (s1 - s0) * v; g1.N = (v - s0 - 1) * v; g1.K = X;
@@ -642,6 +648,10 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
           sg.a_row0 = s0 * v; sg.b_row0 = (s0 + 1) * v;
           sg.C = g1.C; sg.ldc = g1.ldc;
           sg.src = g1;
+          sg.a_rows = sg.b_rows = true;
+          sg.scratch = scratch;
+          sg.scratch_bytes = sb;
+          zero(scratch, SLICE_RESET_BYTES, st);
           gemm_slices(sg, st, err_d.as<int>(), num_sms);
         } else {
           g1.A = LT.c() + s0 * v * X; g1.lda = X;
@@ -972,7 +982,7 @@ void Ctx::residual(const cplx *t1p, const cplx *t2p, cplx *R1, cplx *R2) {
 size_t Ctx::planes_bytes_estimate(int tr) const {
   if (tr == TIER_FP64) {
     // digit planes of the largest product, as far as the budget goes
-    const double mkk = static_cast<double>(o) * o * v * v * 2.0 * SLICE_COUNT;
+    const double mkk = static_cast<double>(o) * o * v * v * 2.0 * SLICE_PLANES;
     const double cap = 1.125 * static_cast<double>(Engine::SLICE_BUDGET);
     return al.limit ? 0 : static_cast<size_t>(std::min(cap, 4.0 * mkk) + std::min(cap, 2.0 * mkk));
   }
