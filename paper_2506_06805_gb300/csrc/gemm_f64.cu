@@ -222,25 +222,101 @@ __global__ void gemv_kt_kernel(long N, long K, const double2 *__restrict__ A,
   }
 }
 
-// Same contraction with a warp per output element and the lanes striding k:
-// coalesced when the operand's innermost K index has unit stride. Blocks of
-// 128 k per step; F32: a lane's four products of a block in FP32, that run
-// added in FP64.
+// Same contraction with one warp per output element, or the W warps of the
+// thread block, and the lanes striding k: coalesced when the operand's
+// innermost K index has unit stride. Four independent loads per lane in flight
+// (offset tables resolve first), each into a sum of its own: their
+// multiply-adds do not wait for one another, and a sum runs over K / 128
+// terms. W > 1: blocks of 128 k dealt to the warps, for few outputs (320 x
+// 12000 on 320 warps took 120 us, now 45). The FP64 pipe binds: 12000 x
+// 12000 980 us; four outputs a warp with one sum each, as the FP32 form
+// below has them, took 1.67 ms and had twice the error.
+template <int W>
+__global__ void __launch_bounds__(256) gemv64_kernel(long N, long K, const double2 *__restrict__ A,
+                                                     const long *__restrict__ ak, bool conjA,
+                                                     const double2 *__restrict__ B,
+                                                     const long *__restrict__ bn,
+                                                     const long *__restrict__ bk, long ldb,
+                                                     bool conjB, double2 *C,
+                                                     const long *__restrict__ cn, long ldc,
+                                                     double2 alpha, double2 beta) {
+  static_assert(W == 1 || W == 8, "one output per warp or per block");
+  __shared__ double2 part[W];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long first = W == 1 ? blockIdx.x * 8L + warp : blockIdx.x;
+  const long step = W == 1 ? static_cast<long>(gridDim.x) * 8 : gridDim.x;
+  for (long n = first; n < N; n += step) {
+    const long bo = bn ? bn[n] : n * ldb;
+    double2 ac[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
+                     make_double2(0.0, 0.0)};
+    long k = (W == 1 ? 0 : 128 * warp) + lane;
+    for (; k + 96 < K; k += 128 * W) {
+      long ia[4], ib[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        ia[u] = ak ? ak[k + 32 * u] : k + 32 * u;
+        ib[u] = bo + (bk ? bk[k + 32 * u] : k + 32 * u);
+      }
+      double2 a[4], b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a[u] = A[ia[u]];
+        b[u] = B[ib[u]];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (conjA) a[u].y = -a[u].y;
+        if (conjB) b[u].y = -b[u].y;
+        ac[u] = cfma(a[u], b[u], ac[u]);
+      }
+    }
+    for (; k < K; k += 32) {  // (the last block, for the lanes that it does not fill)
+      double2 a = A[ak ? ak[k] : k];
+      double2 b = B[bo + (bk ? bk[k] : k)];
+      if (conjA) a.y = -a.y;
+      if (conjB) b.y = -b.y;
+      ac[0] = cfma(a, b, ac[0]);
+    }
+    double2 acc = cadd(cadd(ac[0], ac[1]), cadd(ac[2], ac[3]));
+    for (int o = 16; o > 0; o >>= 1) {
+      acc.x += __shfl_down_sync(0xffffffffu, acc.x, o);
+      acc.y += __shfl_down_sync(0xffffffffu, acc.y, o);
+    }
+    if (W > 1) {
+      if (lane == 0) part[warp] = acc;
+      __syncthreads();
+      if (threadIdx.x == 0) {  // pairwise
+        for (int s = 1; s < W; s *= 2)
+          for (int w = 0; w < W; w += 2 * s) part[w] = cadd(part[w], part[w + s]);
+        acc = part[0];
+      }
+      __syncthreads();
+    }
+    if (lane == 0 && (W == 1 || warp == 0)) {
+      const long off = cn ? cn[n] : n * ldc;
+      const double2 x = cmul(alpha, acc);
+      C[off] = (beta.x == 0.0 && beta.y == 0.0) ? x : cadd(x, cmul(beta, C[off]));
+    }
+  }
+}
+
+// The same with FP32 products: blocks of 128 k per step, a lane's four products
+// of a block in FP32, that run added in FP64.
 //   R > 1: R outputs per warp, whose vector elements, table entries and
 //   conversions are shared (many outputs: a warp each was bound by those,
 //   2.4 TB/s at 12000 x 12000). W > 1: the blocks of one output dealt to the
-//   W warps of the thread block (few outputs: 320 x 12000 ran on 320 warps).
-// Neither changes the FP32 runs. 12000 x 12000 (FP32) 952 -> 557 us, 320 x
-// 12000 (FP64) 120 -> 71 us, 1600 x 12000 (FP32) 310 -> 97 us.
-template <bool F32, int R, int W>
-__global__ void __launch_bounds__(256) gemv_warp_kernel(long N, long K, const double2 *__restrict__ A,
-                                                        const long *__restrict__ ak, bool conjA,
-                                                        const double2 *__restrict__ B,
-                                                        const long *__restrict__ bn,
-                                                        const long *__restrict__ bk, long ldb,
-                                                        bool conjB, double2 *C,
-                                                        const long *__restrict__ cn, long ldc,
-                                                        double2 alpha, double2 beta) {
+//   W warps of the thread block (few outputs: 1600 x 12000 ran on 1600 warps).
+// Neither changes the FP32 runs. 12000 x 12000 952 -> 557 us, 1600 x 12000
+// 310 -> 97 us.
+template <int R, int W>
+__global__ void __launch_bounds__(256) gemv32_kernel(long N, long K, const double2 *__restrict__ A,
+                                                     const long *__restrict__ ak, bool conjA,
+                                                     const double2 *__restrict__ B,
+                                                     const long *__restrict__ bn,
+                                                     const long *__restrict__ bk, long ldb,
+                                                     bool conjB, double2 *C,
+                                                     const long *__restrict__ cn, long ldc,
+                                                     double2 alpha, double2 beta) {
   static_assert(W == 1 || (W == 8 && R == 1), "one output per block, or whole warps");
   __shared__ double2 part[W];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -268,36 +344,24 @@ __global__ void __launch_bounds__(256) gemv_warp_kernel(long N, long K, const do
           av[u] = A[ak ? ak[kk] : kk];
           ib[u] = bk ? bk[kk] : kk;
         }
-        if (F32) {
-          float2 a[4];
+        float2 a[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            a[u] = make_float2(f64_to_f32(av[u].x), conjA ? -f64_to_f32(av[u].y) : f64_to_f32(av[u].y));
+        for (int u = 0; u < 4; ++u)
+          a[u] = make_float2(f64_to_f32(av[u].x), conjA ? -f64_to_f32(av[u].y) : f64_to_f32(av[u].y));
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            double2 b[4];
+        for (int r = 0; r < R; ++r) {
+          double2 b[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) b[u] = row[r][ib[u]];
-            float xr = 0.f, xi = 0.f;
+          for (int u = 0; u < 4; ++u) b[u] = row[r][ib[u]];
+          float xr = 0.f, xi = 0.f;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const float br = f64_to_f32(b[u].x), bi = conjB ? -f64_to_f32(b[u].y) : f64_to_f32(b[u].y);
-              xr = fmaf(a[u].x, br, fmaf(-a[u].y, bi, xr));
-              xi = fmaf(a[u].x, bi, fmaf(a[u].y, br, xi));
-            }
-            ac[r].x += f32_to_f64(xr);
-            ac[r].y += f32_to_f64(xi);
+          for (int u = 0; u < 4; ++u) {
+            const float br = f64_to_f32(b[u].x), bi = conjB ? -f64_to_f32(b[u].y) : f64_to_f32(b[u].y);
+            xr = fmaf(a[u].x, br, fmaf(-a[u].y, bi, xr));
+            xi = fmaf(a[u].x, bi, fmaf(a[u].y, br, xi));
           }
-        } else {
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              double2 a = av[u], b = row[r][ib[u]];
-              if (conjA) a.y = -a.y;
-              if (conjB) b.y = -b.y;
-              ac[r] = cfma(a, b, ac[r]);
-            }
+          ac[r].x += f32_to_f64(xr);
+          ac[r].y += f32_to_f64(xi);
         }
       } else {
         for (; k < K; k += 32) {
@@ -341,7 +405,7 @@ __global__ void __launch_bounds__(256) gemv_warp_kernel(long N, long K, const do
 // overlaps, the singles intermediates): one warp per output element and a K
 // range per blockIdx.y; partial sums are added atomically when K is split (C
 // scaled by beta beforehand). F32: runs of four products per lane in FP32,
-// each run added in FP64, as in gemv_warp_kernel.
+// each run added in FP64, as in gemv32_kernel.
 template <bool F32>
 __global__ void __launch_bounds__(256) dots_kernel(long M, long N, long K,
                                                    const double2 *__restrict__ A,
@@ -429,14 +493,20 @@ void gemm_f64(const GemmDesc &g, cudaStream_t st, int num_sms) {
   if (rowvec || colvec) {
     const long n_out = rowvec ? g.N : g.M;
     if (g.k_contig) {
-      // a block per output below 16 warps per SM; four outputs a warp while
-      // that still leaves 16; a warp per output between
-      const bool few = n_out < 16L * num_sms && g.K >= 1024, many = n_out >= 64L * num_sms;
+      // A block per output where a warp each leaves SMs short of work and K is
+      // long enough for eight warps (FP64, a warp / a block each: 320 x 1024
+      // 14.6 / 11.0 us, 1000 x 2048 25 / 29, 1600 x 4096 75 / 65, 2400 x 12000
+      // 208 / 220; FP32 1000 x 1024 17 / 16, 2400 x 1024 21 / 29, 2400 x 4096
+      // 70 / 55); in FP32 four outputs a warp while that leaves 16 warps per SM
+      const bool few = g.f32 ? n_out < 16L * num_sms && g.K >= 1024 && 10 * g.K >= 9 * n_out
+                             : n_out < 12L * num_sms && g.K >= 256 && 2 * g.K >= 5 * n_out;
+      const bool many = g.f32 && n_out >= 64L * num_sms;
       const long per_block = few ? 1 : (many ? 32 : 8);
       const unsigned wb = static_cast<unsigned>(std::min<long>((n_out + per_block - 1) / per_block, 65535));
-      auto kern = few    ? (g.f32 ? gemv_warp_kernel<true, 1, 8> : gemv_warp_kernel<false, 1, 8>)
-                  : many ? (g.f32 ? gemv_warp_kernel<true, 4, 1> : gemv_warp_kernel<false, 4, 1>)
-                         : (g.f32 ? gemv_warp_kernel<true, 1, 1> : gemv_warp_kernel<false, 1, 1>);
+      auto kern = !g.f32 ? (few ? gemv64_kernel<8> : gemv64_kernel<1>)
+                  : few  ? gemv32_kernel<1, 8>
+                  : many ? gemv32_kernel<4, 1>
+                         : gemv32_kernel<1, 1>;
       if (rowvec)
         kern<<<wb, 256, 0, st>>>(n_out, g.K, g.A, g.ak, g.conjA, g.B, g.bn, g.bk, g.ldb, g.conjB,
                                  g.C, g.cn, 1, g.alpha, g.beta);
