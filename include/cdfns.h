@@ -275,7 +275,10 @@ int cc_set_graphs(cc_ctx *ctx, int on);
  * packed stable operands (otherwise packed again on each use) and a permuted
  * copy of <mb||ej>. The results do not depend on these choices beyond the
  * convergence tolerance. Must not lower the cap below the bytes already held
- * (CC_ERR_ARG). */
+ * (CC_ERR_ARG). FP64 products of a context with a cap run on the FP64 pipe;
+ * without one, their operand planes take up to 4 GiB or an eighth of the free
+ * memory each, stay with the context, and are given back when an allocation
+ * fails. */
 int cc_set_memory_limit(cc_ctx *ctx, size_t bytes);
 
 /* Amplitudes as unique elements, host complex128: t1 [o][v] then t2 for

@@ -48,7 +48,7 @@ void *Allocator::get(size_t bytes) {
       break;
     }
   }
-  for (int attempt = 0; !p; ++attempt) {
+  for (bool reclaimed = false; !p;) {
     if (alloc) {
       p = alloc(bytes, user);
     } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
@@ -56,9 +56,13 @@ void *Allocator::get(size_t bytes) {
       p = nullptr;
     }
     if (p) break;
-    if (attempt == 0 && !held.empty()) {
+    if (!held.empty()) {
       flush_held();  // the kept blocks back to their allocator, then once more
       continue;
+    }
+    if (!reclaimed && reclaim) {
+      reclaimed = true;
+      if (reclaim(reclaim_arg)) continue;
     }
     fail(CC_ERR_OOM, (alloc ? "device allocation of " : "cudaMalloc of ") +
                          std::to_string(bytes) + " bytes failed");

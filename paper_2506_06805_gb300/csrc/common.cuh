@@ -105,6 +105,10 @@ struct Allocator {
     void (*fr)(void *, void *);
     void *fr_user;
   };
+  // Called when an allocation fails, to give back scratch that can be made
+  // again (true if there was any) before the one retry.
+  bool (*reclaim)(void *) = nullptr;
+  void *reclaim_arg = nullptr;
   std::vector<Held> held;
   size_t held_bytes = 0;
   bool recycle = false;

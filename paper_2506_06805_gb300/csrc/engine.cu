@@ -511,6 +511,14 @@ size_t Engine::slice_budget(int which, size_t need) {
   return std::max(held, std::min(SLICE_BUDGET, device_avail(al) / 8));
 }
 
+bool Engine::drop_slices() {
+  if (slices_busy_) return false;
+  size_t n = 0;
+  for (int slot : {SLICE_SLOT_A, SLICE_SLOT_B, SLICE_SLOT_S}) n += planes_.erase(slot);
+  if (n) ++gen;
+  return n > 0;
+}
+
 bool Engine::run_slices(const GemmDesc &g, bool a_rows, bool b_rows) {
   // a capped context keeps the memory its cap was chosen for
   if (al->limit) return false;
@@ -533,6 +541,11 @@ bool Engine::run_slices(const GemmDesc &g, bool a_rows, bool b_rows) {
     for (const long M : {std::min(mb, g.M), (g.M - 1) % mb + 1})
       for (const long N : {std::min(nb, g.N), (g.N - 1) % nb + 1})
         sb = std::max(sb, slice_scratch_bytes(M, N, K, num_sms));
+  struct Busy {
+    bool &b;
+    explicit Busy(bool &x) : b(x) { b = true; }
+    ~Busy() { b = false; }
+  } busy(slices_busy_);
   void *ma, *mbuf, *scratch;
   try {
     ma = plane(SLICE_SLOT_A, slice_bytes(true, mb, kb));

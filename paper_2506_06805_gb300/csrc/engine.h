@@ -108,6 +108,9 @@ class Engine {
   // what is already held in their slot, or up to an eighth of the room left
   // and SLICE_BUDGET
   size_t slice_budget(int which, size_t need);
+  // Give the planes and lists of FP64 products back (they are made again when
+  // next used): false when none are held, or in the middle of such a product.
+  bool drop_slices();
   static constexpr size_t SLICE_BUDGET = size_t(4) << 30;
   static constexpr int SLICE_SLOT_A = 1000, SLICE_SLOT_B = 1001, SLICE_SLOT_S = 1002;
   void clear_cache() {
@@ -165,6 +168,7 @@ class Engine {
   std::map<std::string, Packed> packs_;
   std::set<std::string> uncached_;
   std::map<int, Buf> planes_;
+  bool slices_busy_ = false;
   struct TraceRec {
     std::string label;
     long M, N, K;

@@ -121,6 +121,8 @@ void Ctx::create(int n_occ, int n_virt, int n_aux, const double *eps_host) {
   eng.al = &al;
   eng.st = st;
   eng.num_sms = num_sms;
+  al.reclaim = [](void *e) { return static_cast<Engine *>(e)->drop_slices(); };
+  al.reclaim_arg = &eng;
   eng.trace_init();
   err_d.reset(&al, 64);
   stats_d.reset(&al, 64);
@@ -604,18 +606,38 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
     // otherwise each product makes its own from a K-major copy LT[(a,c)][P]
     Buf LT, LA, LB;
     SlicePlanes pA, pB;
-    if (al.limit == 0 && X <= 65536 && slices_pay(v, vv, X) &&
-        slice_bytes(true, vv, X) <= std::min(Engine::SLICE_BUDGET, device_avail(&al) / 8)) {
-      LA.reset(&al, slice_bytes(true, vv, X));
-      LB.reset(&al, slice_bytes(false, vv, X));
+    auto without_planes = [&] {
+      LA.release();
+      LB.release();
+      LT.reset(&al, sizeof(cplx) * vv * X);
+      eng.permute_into(C1(), T(Lv, "Pac", {X, v, v}), C0(), T(LT.c(), "acP", {v, v, X}));
+    };
+    // f, and when it runs out of memory f again with the planes given up for
+    // the copy, which takes a sixth of them
+    auto or_without_planes = [&](auto &&f) {
+      try {
+        f();
+      } catch (const Error &e) {
+        if (e.code != CC_ERR_OOM || LT.p) throw;
+        without_planes();
+        f();
+      }
+    };
+    if (ladder_plane_bytes() && slice_bytes(true, vv, X) <= device_avail(&al) / 8) {
+      or_without_planes([&] {
+        if (LT.p) return;
+        LA.reset(&al, slice_bytes(true, vv, X));
+        LB.reset(&al, slice_bytes(false, vv, X));
+      });
+    } else {
+      without_planes();
+    }
+    if (LA.p) {
       pA = slice_planes(LA.p, true, vv, X);
       pB = slice_planes(LB.p, false, vv, X);
       SliceOperand l;
       l.src = Lv; l.kt = ptab; l.ld = 1; l.rows = vv; l.rows_unit = true;
       slice_pack(&l, &pA, &l, &pB, X, nullptr, st, num_sms);
-    } else {
-      LT.reset(&al, sizeof(cplx) * vv * X);
-      eng.permute_into(C1(), T(Lv, "Pac", {X, v, v}), C0(), T(LT.c(), "acP", {v, v, X}));
     }
     long a0 = 0;
     Buf Vs, W;
@@ -627,14 +649,17 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
       const long p0 = a0 * v - a0 * (a0 + 1) / 2;
       const long p1 = a1 * v - a1 * (a1 + 1) / 2;
       const long np = p1 - p0;
-      B(Vs, nA * per_a);
-      B(W, np * n_cd);
       const auto ranges = slab_rows(v, a0, nA, X);
       size_t sb = 0;
-      if (LA.p)
+      void *scratch = nullptr;
+      or_without_planes([&] {
+        B(Vs, nA * per_a);
+        B(W, np * n_cd);
+        if (LT.p) return;
         for (const auto &ar : ranges)
           sb = std::max(sb, slice_scratch_bytes((ar.second - ar.first) * v, (v - ar.first - 1) * v, X, num_sms));
-      void *scratch = sb ? eng.plane(Engine::SLICE_SLOT_S, sb) : nullptr;
+        scratch = eng.plane(Engine::SLICE_SLOT_S, sb);
+      });
       for (const auto &ar : ranges) {
         const long s0 = ar.first, s1 = ar.second;
         GemmDesc g1;
@@ -984,7 +1009,8 @@ size_t Ctx::planes_bytes_estimate(int tr) const {
     // digit planes of the largest product, as far as the budget goes
     const double mkk = static_cast<double>(o) * o * v * v * 2.0 * SLICE_PLANES;
     const double cap = 1.125 * static_cast<double>(Engine::SLICE_BUDGET);
-    return al.limit ? 0 : static_cast<size_t>(std::min(cap, 4.0 * mkk) + std::min(cap, 2.0 * mkk));
+    const double lists = static_cast<double>(slab_budget + sizeof(cplx) * mkk / (2 * SLICE_PLANES)) / 50.0;
+    return al.limit ? 0 : static_cast<size_t>(std::min(cap, 4.0 * mkk) + std::min(cap, 2.0 * mkk) + lists);
   }
   // the largest doubles-sized contraction (M K = o^2 v^2, N <= M) packs its
   // A side into 2M x 2K and its B side into N x 2K elements of the tier's
@@ -993,9 +1019,18 @@ size_t Ctx::planes_bytes_estimate(int tr) const {
   return static_cast<size_t>(6.0 * mk * tc_elem_bytes(tr) * (tier_split(tr) ? 2 : 1));
 }
 
+// Device bytes of the digit planes of L that the FP64 ladder would make (0: it
+// works from a K-major copy).
+size_t Ctx::ladder_plane_bytes() const {
+  const long vv = static_cast<long>(v) * v;
+  if (al.limit || X > 65536 || !slices_pay(v, vv, X) || slice_bytes(true, vv, X) > Engine::SLICE_BUDGET) return 0;
+  return slice_bytes(true, vv, X) + slice_bytes(false, vv, X);
+}
+
 size_t Ctx::residual_bytes_estimate() const {
   const double nb2 = static_cast<double>(sizeof(cplx)) * o * o * v * v;
-  const double lvv = static_cast<double>(sizeof(cplx)) * X * v * v;
+  double lvv = static_cast<double>(sizeof(cplx)) * X * v * v;
+  if (res_tier() == TIER_FP64) lvv = std::max(lvv, static_cast<double>(ladder_plane_bytes()));
   return static_cast<size_t>(4 * nb2 + lvv) + planes_bytes_estimate(res_tier()) + slab_budget;
 }
 

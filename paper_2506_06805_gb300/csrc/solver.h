@@ -137,6 +137,7 @@ struct Ctx {
   void ensure_pairs();
   // upper estimate of the scratch planes of the tensor-core operands
   size_t planes_bytes_estimate(int tier) const;
+  size_t ladder_plane_bytes() const;
   // upper estimate of the device bytes one CCSD residual allocates and frees
   // again (tau, tau~, X, W, z, the dressed L, ladder slabs, operand planes)
   size_t residual_bytes_estimate() const;
