@@ -278,7 +278,7 @@ int cc_set_graphs(cc_ctx *ctx, int on);
  * (CC_ERR_ARG). FP64 products of a context with a cap run on the FP64 pipe;
  * without one, their operand planes take up to 4 GiB or an eighth of the free
  * memory each, stay with the context, and are given back when an allocation
- * fails. */
+ * fails or a cap is set. */
 int cc_set_memory_limit(cc_ctx *ctx, size_t bytes);
 
 /* Amplitudes as unique elements, host complex128: t1 [o][v] then t2 for

@@ -636,6 +636,7 @@ int cc_set_graphs(cc_ctx *ctx, int on) {
 
 int cc_set_memory_limit(cc_ctx *ctx, size_t bytes) {
   if (!ctx) return CC_ERR_ARG;
+  if (bytes) ctx->c.eng.drop_slices();  // not used under a cap
   if (bytes && bytes < ctx->c.al.in_use) return CC_ERR_ARG;
   ctx->c.al.limit = bytes;
   return CC_OK;

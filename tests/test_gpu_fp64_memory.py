@@ -1,5 +1,5 @@
 """FP64 work in as much memory as it takes without digit planes: the planes are
-given up when an allocation fails."""
+given up when an allocation fails, and when a cap is set."""
 import numpy as np
 import pytest
 
@@ -85,3 +85,21 @@ def test_fp64_work_fits_where_the_pipe_form_fits(call, slab):
             out.append((r1, r2))
     for a, b in zip(*out):
         assert float((a - b).abs().max()) <= 1e-12 * float(a.abs().max() if a.abs().max() > 0 else 1.0)
+
+
+def test_a_cap_gives_the_planes_back():
+    """The planes do not count against a cap set after FP64 work: one byte
+    above what the context held before it is accepted."""
+    P = _gpu()
+    o, v = 10, 72
+    eps, L, t1, t2 = _inputs(o, v)
+    with P.System(eps, L, n_occ=o, tier="fp64") as s:
+        s.set_memory_limit(1 << 36)  # the work's other lasting buffers, first
+        r1, r2 = torch.zeros_like(t1), torch.zeros_like(t2)
+        s.residual_dev(t1, t2, r1, r2)
+        s.set_memory_limit(0)
+        held = int(s.stats()["device_bytes_held"])
+        s.residual_dev(t1, t2, r1, r2)
+        assert int(s.stats()["device_bytes_held"]) > held
+        s.set_memory_limit(held + 1)
+        assert int(s.stats()["device_bytes_held"]) <= held
