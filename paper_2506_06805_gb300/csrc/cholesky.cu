@@ -30,8 +30,6 @@ namespace cdfns {
 namespace {
 
 constexpr int THREADS = 256;
-constexpr int ROW_LANES = 8;                            // lanes per row of B
-constexpr int BLOCK_ROWS = THREADS / ROW_LANES;         // rows per block and pass
 constexpr long MAX_BLOCKS = 8192;                       // partial maxima
 constexpr int STEP_BATCH = 32;
 constexpr int SMEM_R = 2048;                            // coefficients kept in shared memory
@@ -65,9 +63,10 @@ __device__ __forceinline__ Largest block_largest(Largest m) {
 }
 
 // FIRST: d[q] = sum_s |B[q][s]|^2. Otherwise l = B w, L[q] = l, d[q] -= |l|^2.
-// Eight lanes per row (128 contiguous bytes a load, three shuffles for four
-// rows at once); w in shared memory.
-template <bool FIRST>
+// LANES threads per row of B: 8 (128 contiguous bytes a load, three shuffles
+// for four rows at once), a warp, or the block, so that few rows still fill
+// the SMs; w in shared memory.
+template <bool FIRST, int LANES>
 __global__ void __launch_bounds__(THREADS)
     vector_kernel(const double2 *__restrict__ B, long N, int r, const double2 *__restrict__ w,
                   const long *__restrict__ piv, double2 *__restrict__ L, double *__restrict__ d,
@@ -80,17 +79,17 @@ __global__ void __launch_bounds__(THREADS)
     __syncthreads();
     ws = sw;
   }
-  const int lane = threadIdx.x & (ROW_LANES - 1);
+  constexpr int ROWS = THREADS / LANES;  // per block and pass
+  const int lane = threadIdx.x & (LANES - 1);
   Largest m{-1.0, -1};
-  for (long q0 = blockIdx.x * static_cast<long>(BLOCK_ROWS); q0 < N;
-       q0 += static_cast<long>(gridDim.x) * BLOCK_ROWS) {
-    const long q = q0 + threadIdx.x / ROW_LANES;
+  for (long q0 = blockIdx.x * static_cast<long>(ROWS); q0 < N; q0 += static_cast<long>(gridDim.x) * ROWS) {
+    const long q = q0 + threadIdx.x / LANES;
     double xr = 0.0, xi = 0.0;
     if (q < N) {
       const double2 *row = B + q * r;
       double yr = 0.0, yi = 0.0;
 #pragma unroll 4
-      for (int s = lane; s < r; s += ROW_LANES) {
+      for (int s = lane; s < r; s += LANES) {
         const double2 b = row[s];
         if (FIRST) {
           xr = fma(b.x, b.x, xr);
@@ -106,9 +105,21 @@ __global__ void __launch_bounds__(THREADS)
       xr += yr;
       xi += yi;
     }
-    for (int o = ROW_LANES / 2; o > 0; o >>= 1) {
+    for (int o = (LANES < 32 ? LANES : 32) / 2; o > 0; o >>= 1) {
       xr += __shfl_xor_sync(0xffffffffu, xr, o);
       if (!FIRST) xi += __shfl_xor_sync(0xffffffffu, xi, o);
+    }
+    if (LANES > 32) {  // the block's warps, pairwise
+      __shared__ double2 part[THREADS / 32];
+      if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_double2(xr, xi);
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        for (int s = 1; s < THREADS / 32; s *= 2)
+          for (int g = 0; g < THREADS / 32; g += 2 * s) part[g] = cadd(part[g], part[g + s]);
+        xr = part[0].x;
+        xi = part[0].y;
+      }
+      __syncthreads();
     }
     if (q < N && lane == 0) {
       double x;
@@ -176,13 +187,19 @@ __global__ void __launch_bounds__(THREADS)
 
 int pivoted_cholesky(const cplx *B, long N, int r, double tau, int max_vec, cplx *L, long *piv,
                      Allocator *al, cudaStream_t st, int num_sms) {
-  (void)num_sms;
-  const long nb = std::min<long>(MAX_BLOCKS, (N + BLOCK_ROWS - 1) / BLOCK_ROWS);
+  // a step in us with 8 / 32 / 256 threads a row: 300 x 2100 98 / 40 / 24,
+  // 1000 x 1000 54 / 30 / 38, 1000 x 4000 182 / 61 / 57, 2500 x 100 20 / 30 / 44,
+  // 5000 x 800 74 / 68 / 100
+  const int lanes = N > 16L * num_sms ? 8 : N > 2L * num_sms ? 32 : THREADS;
+  auto first = lanes == 8 ? vector_kernel<true, 8> : lanes == 32 ? vector_kernel<true, 32> : vector_kernel<true, THREADS>;
+  auto next = lanes == 8 ? vector_kernel<false, 8> : lanes == 32 ? vector_kernel<false, 32> : vector_kernel<false, THREADS>;
+  const long rows = THREADS / lanes;
+  const long nb = std::min<long>(MAX_BLOCKS, (N + rows - 1) / rows);
   const unsigned grid = static_cast<unsigned>(nb);
   Buf d(al, sizeof(double) * N), W(al, sizeof(cplx) * max_vec * r);
   Buf bv(al, sizeof(double) * nb), bi(al, sizeof(long) * nb), pv(al, sizeof(long) * max_vec);
-  vector_kernel<true><<<grid, THREADS, 0, st>>>(B, N, r, nullptr, nullptr, nullptr, d.as<double>(),
-                                                bv.as<double>(), bi.as<long>());
+  first<<<grid, THREADS, 0, st>>>(B, N, r, nullptr, nullptr, nullptr, d.as<double>(), bv.as<double>(),
+                                  bi.as<long>());
   LAUNCH_CHECK();
   count_launch();
   std::vector<long> hp(max_vec);
@@ -193,9 +210,9 @@ int pivoted_cholesky(const cplx *B, long N, int r, double tau, int max_vec, cplx
       pivot_kernel<<<static_cast<unsigned>((r + 31) / 32), THREADS, 0, st>>>(
           B, N, r, tau, k, nb, bv.as<double>(), bi.as<long>(), L, W.c(), pv.as<long>());
       LAUNCH_CHECK();
-      vector_kernel<false><<<grid, THREADS, 0, st>>>(B, N, r, W.c() + static_cast<long>(k) * r,
-                                                     pv.as<long>() + k, L + static_cast<long>(k) * N,
-                                                     d.as<double>(), bv.as<double>(), bi.as<long>());
+      next<<<grid, THREADS, 0, st>>>(B, N, r, W.c() + static_cast<long>(k) * r, pv.as<long>() + k,
+                                     L + static_cast<long>(k) * N, d.as<double>(), bv.as<double>(),
+                                     bi.as<long>());
       LAUNCH_CHECK();
       count_launch(2);
     }

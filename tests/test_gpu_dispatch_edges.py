@@ -27,3 +27,20 @@ def test_fp64_products_of_8_to_31_terms(M, N, K):
     P.zgemm_dev(A, B, C, "fp64")
     tol = 8 * K * 2.0 ** -53 * (A.abs() @ B.abs().T)
     assert bool(((C - A @ B.T).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("N,r,n", [(304, 70, 50), (305, 70, 50), (1000, 2100, 60), (2432, 33, 20), (2433, 33, 20)])
+def test_pivoted_cholesky_threads_per_row(N, r, n):
+    """A block, a warp or eight threads per row of the generator, against the
+    oracle; its condition is that of a random matrix with 3/4 of its rank taken
+    (remainders above 1e-2 of the diagonal), so FP64 sums of r terms agree to
+    far below 1e-11."""
+    from oracle import cholesky
+    P = _gpu()
+    rng = np.random.default_rng(N + r)
+    B = rng.standard_normal((N, r)) + 1j * rng.standard_normal((N, r))
+    n = min(n, 3 * r // 4)
+    ref, piv_ref = cholesky.pivoted_cholesky(B, 0.0, max_vec=n)
+    L, piv = P.cholesky_dev(torch.from_numpy(B).cuda(), 0.0, n)
+    assert np.array_equal(piv, piv_ref)
+    assert np.abs(L.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max()
