@@ -543,19 +543,33 @@ namespace {
 // at o = 20, v = 160, X = 640 8.29 -> 7.39 ms, at o = 40, v = 300, X = 1200
 // 107.8 -> 105.2 ms. The values of the computed elements do not change.
 //
-// f64_aux != 0: one FP64 launch per range over f64_aux auxiliary indices, so a
-// range costs whole waves of the 76 CTA pairs (K blocks of 32 complex, three
-// for a tile's epilogue) and a launch (two K blocks' time).
-std::vector<std::pair<long, long>> slab_rows(long v, long a0, long nA, long f64_aux = 0) {
+// Less than one wave of units is not split further: a range costs the host its
+// tensor maps and the launch its tile queue (TF32 ladder at o = 6, v = 24, split /
+// not: 167 / 156 us, 58 / 49 of them kernels).
+//
+// FP64 over X auxiliary indices, a launch per range. Digits: whole waves of the
+// CTA pairs (K blocks of 32 complex, three for a tile's epilogue) and a launch
+// (two K blocks' time). Pipe: whole waves of 64 x 64 tiles, 4.2 us a k, or 14
+// ns per 1000 multiply-adds where few tiles make it a warp per output, and a
+// launch (one k's time).
+enum class Slab { TensorCore, Digits, Pipe };
+std::vector<std::pair<long, long>> slab_rows(long v, long a0, long nA, Slab kind, long X, int num_sms) {
+  const long pairs = num_sms / 2;
   auto cost = [&](long s0, long s1) {
-    const long m = (2 * (s1 - s0) * v + 255) / 256;
-    if (!f64_aux) return m * (((v - s0 - 1) * v + 255) / 256);
-    return (m * (((v - s0 - 1) * v + 127) / 128) + 75) / 76 * ((f64_aux + 31) / 32 + 3) + 2;
+    const long M = (s1 - s0) * v, N = (v - s0 - 1) * v, m = (2 * M + 255) / 256;
+    if (kind == Slab::TensorCore) return static_cast<double>(m * ((N + 255) / 256));
+    if (kind == Slab::Digits)
+      return static_cast<double>((m * ((N + 127) / 128) + pairs - 1) / pairs * ((X + 31) / 32 + 3) + 2);
+    const long tiles = (M + 63) / 64 * ((N + 63) / 64);
+    if (tiles < num_sms && M * N <= 65535L * 8) return 1.0 + 3.3e-6 * M * N * X;
+    return 1.0 + static_cast<double>((tiles + num_sms - 1) / num_sms * X);
   };
-  long best = -1, best_n = 1;
+  double best = -1;
+  long best_n = 1;
   for (long n = 1; n <= std::min<long>(TC_MAX_PROBLEMS, nA); ++n) {
-    long u = 0;
+    double u = 0;
     for (long q = 0; q < n; ++q) u += cost(a0 + nA * q / n, a0 + nA * (q + 1) / n);
+    if (kind == Slab::TensorCore) u = std::max(u, static_cast<double>(pairs));
     if (best < 0 || u < best) {
       best = u;
       best_n = n;
@@ -649,12 +663,13 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
       const long p0 = a0 * v - a0 * (a0 + 1) / 2;
       const long p1 = a1 * v - a1 * (a1 + 1) / 2;
       const long np = p1 - p0;
-      const auto ranges = slab_rows(v, a0, nA, X);
+      std::vector<std::pair<long, long>> ranges;
       size_t sb = 0;
       void *scratch = nullptr;
       or_without_planes([&] {
         B(Vs, nA * per_a);
         B(W, np * n_cd);
+        ranges = slab_rows(v, a0, nA, al.limit ? Slab::Pipe : Slab::Digits, X, num_sms);
         if (LT.p) return;
         for (const auto &ar : ranges)
           sb = std::max(sb, slice_scratch_bytes((ar.second - ar.first) * v, (v - ar.first - 1) * v, X, num_sms));
@@ -761,7 +776,7 @@ void Ctx::ladder(const cplx *Lv, const cplx *tau, cplx *R2, int tr, const float 
         Engine::Region r = eng.region("ladder gemm1");
         gemm_tc_tune(&g1, st, err_d.as<int>());
         std::vector<TcDesc> parts;
-        for (const auto &ar : slab_rows(v, a0, nA)) {
+        for (const auto &ar : slab_rows(v, a0, nA, Slab::TensorCore, X, num_sms)) {
           const long s0 = ar.first, s1 = ar.second;
           TcDesc g = g1;
           g.M = (s1 - s0) * v; g.N = (v - s0 - 1) * v;
