@@ -161,20 +161,20 @@ def _check(rc, ctx=None, ok=(0,)):
 
 
 _TORCH_HOOKS = None
+_TORCH_STREAM = None
 
 
 def use_torch_memory():
     """Route the library's device allocations through PyTorch's caching
     allocator and issue its work on torch's current stream."""
-    global _TORCH_HOOKS
+    global _TORCH_HOOKS, _TORCH_STREAM
     import torch
     if not torch.cuda.is_available():
         raise RuntimeError("a CUDA device is required")
-    dev = torch.cuda.current_device()
 
     def _alloc(n, _user):
         try:
-            return torch.cuda.caching_allocator_alloc(int(n), dev)
+            return torch.cuda.caching_allocator_alloc(int(n), torch.cuda.current_device())
         except RuntimeError:
             return None
 
@@ -183,8 +183,9 @@ def use_torch_memory():
 
     hooks = (_ALLOC(_alloc), _FREE(_free))
     _check(lib().cc_set_default_allocator(hooks[0], hooks[1], None))
-    _check(lib().cc_set_default_stream(torch.cuda.current_stream().cuda_stream))
-    _TORCH_HOOKS = hooks
+    stream = torch.cuda.current_stream()
+    _check(lib().cc_set_default_stream(stream.cuda_stream))
+    _TORCH_HOOKS, _TORCH_STREAM = hooks, stream
 
 
 def zgemm_dev(A, B, C, tier="fp64"):
@@ -192,8 +193,17 @@ def zgemm_dev(A, B, C, tier="fp64"):
     t = TIERS[tier] if isinstance(tier, str) else int(tier)
     M, K = A.shape
     N = B.shape[0]
-    _check(lib().cc_zgemm_dev(t, M, N, K, _P(A.data_ptr()), _P(B.data_ptr()),
-                              _P(C.data_ptr())))
+    args = t, M, N, K, _P(A.data_ptr()), _P(B.data_ptr()), _P(C.data_ptr())
+    if _TORCH_STREAM is not None:
+        import torch
+        if (torch.cuda.current_device() == _TORCH_STREAM.device_index
+                and torch.cuda.current_stream() != _TORCH_STREAM):
+            # torch serves a block of its current stream's pool, on which work
+            # may be pending; the library works on the stream it was given
+            with torch.cuda.stream(_TORCH_STREAM):
+                _check(lib().cc_zgemm_dev(*args))
+            return
+    _check(lib().cc_zgemm_dev(*args))
 
 
 def batch_ipeom(systems, n_roots, tol=1e-7, max_iter=100, allow_unconverged=False):
