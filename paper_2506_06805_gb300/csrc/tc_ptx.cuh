@@ -126,9 +126,13 @@ __device__ __forceinline__ uint32_t leader_addr(uint32_t a) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
   return r;
 }
-// arrive on an mbarrier given by its shared::cluster address
+// Arrive on an mbarrier given by its shared::cluster address, in the cluster's
+// scope (the default is the CTA's). Relaxed: what the other CTA waits for is
+// reads of the accumulator, which tcgen05.fence::before_thread_sync orders; a
+// release also waits for this thread's stores (the FP64 digit products then
+// take 1.6 times as long).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t a) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
 }
 // TMA load into this CTA's shared memory whose completion is counted on the
 // barrier at shared::cluster address bar (the leader's, in a CTA pair)
