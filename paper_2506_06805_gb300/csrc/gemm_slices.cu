@@ -117,7 +117,7 @@ __device__ __noinline__ void fix_push(const FixList &x, long pt, unsigned left) 
 
 struct alignas(64) SliceArgs {
   CUtensorMap mA, mB;  // [slice][row][Kp] planes as one matrix of slice * rows rows
-  long M, N;           // complex rows, columns of this product
+  long M, N, K;        // complex rows, columns, terms of this product
   long rows_a, rows_b; // plane rows per slice
   long a_row0, b_row0; // first plane row of this product
   const int *ea, *eb;  // per complex row: biased exponent of the largest magnitude
@@ -540,7 +540,10 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
       // mask, left to slice_fix_kernel. S = 0 has no nonzero term: 0 exactly.
       unsigned left;
       {
-        const float rk = sqrtf(32.0f * static_cast<float>(nkb));
+        // (sqrt(K); a shorter last split may have that much less: the others
+        // make up for it)
+        const float full = static_cast<float>(min(P.K, 32L * P.kb_per_split));
+        const float rk = static_cast<float>(min(P.K - 32L * kb0, 32L * nkb)) * rsqrtf(full);
         const float thr = 0x1p30f * rk * (u ? fmaxf(0x1p-4f, 0x1p-8f * rk) : 0x1p-7f);
         left = 0;
         const int buf = bq.pop();
@@ -1261,6 +1264,7 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
   SliceArgs a = {};
   a.M = g.M;
   a.N = g.N;
+  a.K = g.src.K;
   a.rows_a = A.plane_rows;
   a.rows_b = B.plane_rows;
   a.a_row0 = 2 * g.a_row0;
