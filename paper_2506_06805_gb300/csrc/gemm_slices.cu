@@ -1341,16 +1341,17 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
 // Estimated times (s) of an M x N x K product here and on the FP64 pipe. The
 // tensor side: 29 products of every 128 x 128 x 64 block at about 1
 // PF/s, an epilogue of three K blocks per tile, the planes written and read,
-// five launches. The FP64 side: 1 TF/s or its operands at 5 TB/s, on whole
+// five launches per block of 65536 k (8 x 64 x 300000, five blocks: 1.87 ms,
+// 1.21 on the FP64 pipe). The FP64 side: 1 TF/s or its operands at 5 TB/s, on whole
 // 64 x 64 tiles where the tiled kernel takes the product (a tile's rows cost
 // the same empty: 5 x 64000 x 160 took 4.5 ms there).
 bool slices_pay(long M, long N, long K) {
   const double m = (2 * M + 127) / 128 * 128.0, n = (N + 127) / 128 * 128.0;
   const double kb = static_cast<double>((2 * K + 63) / 64);
-  const double mma = 2.0 * m * n * 64.0 * 29.0 * (kb + 3.0) / 1e15;
-  const double pack = (static_cast<double>(M) * K * (32 + 128) + static_cast<double>(N) * K * (32 + 64)) / 5e12;
+  const double mma = 2.0 * m * n * 64.0 * 29.0 * (kb + 3.0) / 1.04e15;
+  const double pack = (static_cast<double>(M) * K * (32 + 128) + static_cast<double>(N) * K * (32 + 64)) / 5.5e12;
   const double out = 32.0 * M * N / 5e12;
-  const double t_slices = 20e-6 + std::max(mma, 20e-6) + pack + out;
+  const double t_slices = 20e-6 * ((K + 65535) / 65536) + std::max(mma, 20e-6) + pack + out;
   const long tm = (M + 63) / 64, tn = (N + 63) / 64;
   const bool skinny = K <= SKINNY64_MAX_K && std::min(M, N) <= 256 && std::max(M, N) >= 1024;
   const bool tiled = M > 1 && N > 1 && !skinny && tm * tn >= 152;
