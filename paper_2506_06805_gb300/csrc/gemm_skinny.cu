@@ -191,22 +191,49 @@ __global__ void __launch_bounds__(SK_THREADS) skinny64_kernel(const SkinnyDesc d
   }
 }
 
-// Short rows per block: as many as the shared memory takes, unless the long
-// side leaves fewer than about four blocks per SM: then the short side is cut
-// as well, down to min_s rows (each block reads its long rows again, from L2).
-// One block row per 256 long rows had left a K = 1 product of 3200 x 100 on 13
-// SMs (236 us, now 15); FP64 residual at o = 10, v = 30, X = 120 2.83 -> 1.95
-// ms, FP16 residual at o = 40, v = 300, X = 1200 102.8 -> 100.6 ms.
-int pick_chunk(const SkinnyDesc &d, int per_s, int min_s, int *ny) {
+// Short rows per block (and blocks along them, ny): as many as the shared
+// memory takes, unless fewer leave clearly less work to the busiest SM (by 5 %
+// in FP64, 15 % in FP32, as far as the estimate can tell). A block costs its
+// short rows and about half of one (FP64) or eight (FP32) more for reading its
+// long rows, again from L2. One block row per 256 long rows had left a K
+// = 1 product of 3200 x 100 on 13 SMs (236 us, now 15); splitting wherever an SM
+// had fewer than four blocks took 16.9 us instead of 11.0 for 60000 rows x 9
+// outputs, K = 16, in FP32, and 88.7 instead of 78.2 for 60000 x 4, K = 32, in
+// FP64. FP64 residual at o = 10, v = 30, X = 120 2.83 -> 1.95 ms, FP16 residual
+// at o = 40, v = 300, X = 1200 102.8 -> 100.6 ms.
+int pick_chunk(const SkinnyDesc &d, int per_s, int *ny) {
+  static const long sms = [] {
+    int dev = 0, n = 0;
+    CUDA_CHECK(cudaGetDevice(&dev));
+    CUDA_CHECK(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return static_cast<long>(n);
+  }();
   const long bx = (d.Mb + SK_THREADS - 1) / SK_THREADS;
-  const int cap = std::max(1, std::min(d.Ns, SK_SMEM / per_s));
-  const long want = std::min<long>((d.Ns + min_s - 1) / min_s, (4L * 152 + bx - 1) / bx);
+  // (even: the FP32 kernel takes two short rows a pass)
+  const int cap = std::max(1, std::min(d.Ns, SK_SMEM / per_s / 2 * 2));
+  const double reload = d.f64 ? 0.5 : 8.0;
+  // the busiest SM's rows with n blocks along c short rows each, rem the last
+  // one's (those of the last ones fill up the other SMs)
+  auto cost = [&](long n, long c) {
+    const long rem = d.Ns - (n - 1) * c, full = rem == c ? n : n - 1;
+    const double busiest = static_cast<double>((bx * full + sms - 1) / sms) * (reload + c);
+    if (rem == c) return busiest;
+    return std::max(busiest, static_cast<double>(bx) / sms * (d.Ns + n * reload) + 0.5 * (rem + reload));
+  };
   int chunk = cap;
-  if (want > (d.Ns + cap - 1) / cap) {
-    chunk = static_cast<int>((d.Ns + want - 1) / want);
-    chunk += chunk & 1;  // the FP32 kernel takes two short rows a pass
+  *ny = 1;
+  double best = cost(1, d.Ns) * (d.f64 ? 0.95 : 0.85);
+  // (FP64: the finest split into pairs of rows up to four blocks per SM)
+  const long most = std::min<long>((d.Ns + 1) / 2, (4 * sms + bx - 1) / bx);
+  for (long n = d.f64 ? most : 2; n >= 2 && n <= most; ++n) {
+    int c = static_cast<int>((d.Ns + n - 1) / n);
+    c += c & 1;
+    const long blocks = (d.Ns + c - 1) / c;
+    if (c > cap || blocks < 2 || blocks > 65535 || cost(blocks, c) >= best) continue;
+    best = cost(blocks, c);
+    chunk = c;
+    *ny = static_cast<int>(blocks);
   }
-  *ny = static_cast<int>(std::min<long>(bx >= 4L * 152 ? 1 : (d.Ns + chunk - 1) / chunk, 65535));
   return chunk;
 }
 
@@ -221,7 +248,7 @@ void skinny_launch(const SkinnyDesc &d, cudaStream_t st) {
   (void)attr;
   const int per_s = (KM / 2) * static_cast<int>(sizeof(float4));
   int ny;
-  const int chunk = pick_chunk(d, per_s, 8, &ny);
+  const int chunk = pick_chunk(d, per_s, &ny);
   const int beta_mode = (d.beta.x == 0.0 && d.beta.y == 0.0) ? 0
                         : (d.beta.x == 1.0 && d.beta.y == 0.0) ? 1
                                                                : 2;
@@ -244,7 +271,7 @@ void skinny64_launch(const SkinnyDesc &d, cudaStream_t st) {
   (void)attr;
   const int per_s = KM * static_cast<int>(sizeof(double2));
   int ny;
-  const int chunk = pick_chunk(d, per_s, 2, &ny);
+  const int chunk = pick_chunk(d, per_s, &ny);
   const long blocks = (d.Mb + SK_THREADS - 1) / SK_THREADS;
   skinny64_kernel<KM><<<dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(ny)), SK_THREADS,
                         chunk * per_s, st>>>(d, chunk);

@@ -44,3 +44,19 @@ def test_pivoted_cholesky_threads_per_row(N, r, n):
     L, piv = P.cholesky_dev(torch.from_numpy(B).cuda(), 0.0, n)
     assert np.array_equal(piv, piv_ref)
     assert np.abs(L.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("M,N,K,tier", [(20000, 41, 33, "fp16x3"), (40000, 100, 32, "fp16x3"), (9000, 9, 40, "fp16x3"),
+                                        (60000, 9, 16, "fp16x3"), (2100, 1000, 40, "fp16x3"),
+                                        (40000, 4, 8, "fp64"), (20000, 4, 16, "fp64"), (5000, 250, 2, "fp64")])
+def test_short_k_products_whole_or_cut(M, N, K, tier):
+    """The short side whole or cut over blocks: sums of 2 K products in FP32
+    (2 K 2^-24) or FP64 (2 K 2^-53), against the sum of their magnitudes."""
+    P = _gpu()
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    cn = lambda *s: torch.view_as_complex(torch.randn(*s, 2, generator=g, device="cuda", dtype=torch.float64))
+    A, B = cn(M, K), cn(N, K)
+    C = torch.empty((M, N), dtype=torch.complex128, device="cuda")
+    P.zgemm_dev(A, B, C, tier)
+    tol = 8 * K * 2.0 ** (-53 if tier == "fp64" else -24) * (A.abs() @ B.abs().T)
+    assert bool(((C - A @ B.T).abs() <= tol).all())
