@@ -1351,7 +1351,10 @@ bool slices_pay(long M, long N, long K) {
   const double mma = 2.0 * m * n * 64.0 * 29.0 * (kb + 3.0) / 1.04e15;
   const double pack = (static_cast<double>(M) * K * (32 + 128) + static_cast<double>(N) * K * (32 + 64)) / 5.5e12;
   const double out = 32.0 * M * N / 5e12;
-  const double t_slices = 20e-6 * ((K + 65535) / 65536) + std::max(mma, 20e-6) + pack + out;
+  // (few outputs: K is split over many SMs, whose additions to the output cost
+  // 10 us more; 30 x 30 x 10000 95 us, 85 on the FP64 pipe)
+  const double few = M * N <= 4096 ? 10e-6 : 0.0;
+  const double t_slices = 20e-6 * ((K + 65535) / 65536) + few + std::max(mma, 20e-6) + pack + out;
   const long tm = (M + 63) / 64, tn = (N + 63) / 64;
   const bool skinny = K <= SKINNY64_MAX_K && std::min(M, N) <= 256 && std::max(M, N) >= 1024;
   const bool tiled = M > 1 && N > 1 && !skinny && tm * tn >= 152;
