@@ -33,13 +33,17 @@
 // A meet small ones of B (columns scaled one way in A and the other in B,
 // sparse rows, small imaginary parts). So an eighth plane holds the rounded
 // magnitudes, whose product, one more beside the 28, gives S of every real and
-// imaginary part, and elements with 0 < S < 2^-7 sqrt(K) 2^(Ea + Eb) are not
-// stored but listed for slice_fix_kernel (where group 5 is in FP32, whose error
-// grows by another 2^-63.8 K 2^(Ea + Eb), those below the larger of 2^-4 sqrt(K)
-// and 2^-8 K), which computes them on the FP64 pipe. So are the elements
+// imaginary part, and elements with 0 < S < t sqrt(K) 2^(Ea + Eb) are not stored
+// but listed for slice_fix_kernel (where group 5 is in FP32, whose error grows
+// by another 2^-63.8 K 2^(Ea + Eb), those below the larger of 8 t sqrt(K) and t K
+// / 2). t is 2^-8.5, where the digits' error reaches 0.38 RMS and 1.4 at most in
+// units of 2^-53 S, that of the FP64 tiles being 0.45 and 2.2, and 2^-7 (0.13)
+// for the few outputs that the FP64 pipe would sum by warps. With 2^-7 for all
+// an FP64 CCSD iteration at o = 40, v = 300, X = 1200 takes 3.3 s, 2.4 so, 2.37
+// with nothing listed. That kernel computes them on the FP64 pipe. So are the elements
 // of rows with an Inf or NaN, which cannot be cut. RMS error over S in units of
 // 2^-53 (1536 x 1000 x 1200, here / FP64 kernel): normal operands 0.024 / 0.47,
-// columns scaled by 10^(+-2 k / K) 0.045 / 0.47, by 10^(+-3 k / K) and more
+// columns scaled by 10^(+-2 k / K) 0.045 / 0.47, by 10^(+-4 k / K) and more
 // (every element listed) 0.071 / 0.47, where it takes 15.3 ms against 14.7 on
 // the FP64 pipe alone and 0.59 with none listed.
 #include <cuda_fp16.h>
@@ -123,6 +127,7 @@ struct alignas(64) SliceArgs {
   const int *ea, *eb;  // per complex row: biased exponent of the largest magnitude
   const float *na, *nb;  // per complex row: squared 2-norm over 4^E
   FixList fix;           // elements left to slice_fix_kernel
+  float least;           // S / sqrt(K) they lie below (over 2^(Ea + Eb))
   double2 *C;
   const long *cm, *cn;
   long ldc;
@@ -544,7 +549,7 @@ __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __gr
         // make up for it)
         const float full = static_cast<float>(min(P.K, 32L * P.kb_per_split));
         const float rk = static_cast<float>(min(P.K - 32L * kb0, 32L * nkb)) * rsqrtf(full);
-        const float thr = 0x1p30f * rk * (u ? fmaxf(0x1p-4f, 0x1p-8f * rk) : 0x1p-7f);
+        const float thr = 0x1p30f * rk * P.least * (u ? fmaxf(8.0f, 0.5f * rk) : 1.0f);
         left = 0;
         const int buf = bq.pop();
         drain(buf, [&](int j, const float (&x)[16]) {
@@ -1310,6 +1315,10 @@ void gemm_slices(const SliceGemm &g, cudaStream_t st, int *err, int num_sms) {
     scale_2d(g.C, g.cm, g.cn, g.ldc, g.M, g.N, g.beta, st);
     a.wmode = SW_ADD;
   }
+  // (the rule of gemm_f64 for outputs that warps sum, in short chains; its
+  // tiles sum K terms one after another)
+  const long tiles = (g.M + 63) / 64 * ((g.N + 63) / 64);
+  a.least = tiles < num_sms && g.M * g.N <= 65535L * 8 ? 0x1p-7f : 0x1.6ap-9f;
   const int u = static_cast<int>(p.units());
   if (p.pair) launch_slices<4, true>(a, A, B, u, num_sms, st);
   else launch_slices<3, false>(a, A, B, u, num_sms, st);
