@@ -496,7 +496,7 @@ int cc_zgemm_dev(int tier, long M, long N, long K, const double *A, const double
     // cudaMalloc and cudaFree, which synchronise, into a lookup. Per call, with
     // torch's allocator / with cudaMalloc: FP16 209 x 171 x 222 83 / 204 us (74
     // where the driver holds free pages from earlier blocks), FP64
-    // 209 x 171 x 222 130 / 297, 1536 x 1000 x 1200 560 / 870.
+    // 209 x 171 x 222 142 / 301, 1536 x 1000 x 1200 577 / 887.
     cdfns::Allocator al;
     {
       std::lock_guard<std::mutex> lk(cdfns::g_mu);

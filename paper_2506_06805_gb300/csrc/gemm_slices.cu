@@ -20,32 +20,31 @@
 // group 5 joins the FP32 part. The sum may wrap on the way, only its value
 // counts.
 //
-// Accuracy, RMS error over |a_m| |b_n| against quadruple precision, here and
-// from the FP64 kernel, normal operands: K = 160 7.9e-18 / 1.3e-17, K = 1200
-// 2.7e-18 / 6.0e-18, K = 20000 1.1e-18 / 4.3e-18.
+// Accuracy, RMS error over |a_m| |b_n| against twice the precision, here and
+// from the FP64 kernel, normal operands: K = 160 5.7e-18 / 1.2e-17, K = 1200
+// 2.4e-18 / 5.8e-18, K = 20000 0.9e-18 / 4.2e-18.
 //
-// Measured against the FP64 kernels: product of 1536 x 1000 x 1200 14.7 ->
-// 0.57 ms, ladder at o = 15, v = 131, X = 517 983 -> 21 ms, FP64 residual at
-// o = 12, v = 72, X = 288 80.7 -> 5.1 ms.
+// The digits' error is relative to the rows' largest magnitudes, FP64's (2^-55
+// to 2^-54 RMS) to S = sum_k |a_mk| |b_nk|, which is far smaller where large
+// elements of A meet small ones of B (columns scaled one way in A and the
+// other in B, sparse rows, small imaginary parts). So an eighth plane holds
+// the rounded magnitudes, whose product, one more beside the 28, gives S of
+// every real and imaginary part. Elements with 0 < S < t sqrt(K) 2^(Ea + Eb)
+// are not stored but listed for slice_fix_kernel, which computes them on the
+// FP64 pipe; so are the elements of rows with an Inf or NaN, which cannot be
+// cut. (Where group 5 is in FP32, whose error grows by another 2^-63.8 K
+// 2^(Ea + Eb), the line is the larger of 8 t sqrt(K) and t K / 2.) t is 2^-8.5,
+// where the digits' error reaches 0.38 RMS and 1.4 at most in units of 2^-53 S,
+// that of the FP64 tiles being 0.45 and 2.2, and 2^-7 (0.13) for the few
+// outputs that the FP64 pipe would sum by warps. 2^-7 for all: an FP64 CCSD
+// iteration at o = 40, v = 300, X = 1200 takes 3.3 s instead of 2.4.
 //
-// That error is relative to the rows' largest magnitudes, FP64's (2^-55 to 2^-54
-// RMS) to S = sum_k |a_mk| |b_nk|, which is far smaller where large elements of
-// A meet small ones of B (columns scaled one way in A and the other in B,
-// sparse rows, small imaginary parts). So an eighth plane holds the rounded
-// magnitudes, whose product, one more beside the 28, gives S of every real and
-// imaginary part, and elements with 0 < S < t sqrt(K) 2^(Ea + Eb) are not stored
-// but listed for slice_fix_kernel (where group 5 is in FP32, whose error grows
-// by another 2^-63.8 K 2^(Ea + Eb), those below the larger of 8 t sqrt(K) and t K
-// / 2). t is 2^-8.5, where the digits' error reaches 0.38 RMS and 1.4 at most in
-// units of 2^-53 S, that of the FP64 tiles being 0.45 and 2.2, and 2^-7 (0.13)
-// for the few outputs that the FP64 pipe would sum by warps. With 2^-7 for all
-// an FP64 CCSD iteration at o = 40, v = 300, X = 1200 takes 3.3 s, 2.4 so, 2.37
-// with nothing listed. That kernel computes them on the FP64 pipe. So are the elements
-// of rows with an Inf or NaN, which cannot be cut. RMS error over S in units of
-// 2^-53 (1536 x 1000 x 1200, here / FP64 kernel): normal operands 0.024 / 0.47,
-// columns scaled by 10^(+-2 k / K) 0.045 / 0.47, by 10^(+-4 k / K) and more
-// (every element listed) 0.071 / 0.47, where it takes 15.3 ms against 14.7 on
-// the FP64 pipe alone and 0.59 with none listed.
+// RMS error over S in units of 2^-53 at 1536 x 1000 x 1200, here / FP64 kernel:
+// normal operands 0.024 / 0.47, columns scaled by 10^(+-2 k / K) 0.045 / 0.47,
+// by 10^(+-4 k / K) and more, where every element is listed, 0.071 / 0.47.
+// That product takes 0.59 ms with none listed, 15.3 with all; 14.7 on the FP64
+// pipe alone. Ladder at o = 15, v = 131, X = 517 983 -> 21.7 ms, FP64 residual
+// at o = 12, v = 72, X = 288 80.7 -> 5.4 ms.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -206,7 +205,8 @@ __device__ __forceinline__ double i64_to_f64(long long t) {
   return __longlong_as_double(static_cast<long long>(b | s));
 }
 
-// The order of the digit products, shared by the three roles. Groups go in
+// The order of the digit products, shared by the three roles, after that of
+// the magnitudes (one accumulation over all K blocks). Groups go in
 // pairs (G, G - 1) for G = 7, 5, 3, 1, and within a K block the 2 G - 1
 // products of such a pair zigzag through the digits,
 //   (A_1, B_G), (A_1, B_G-1), (A_2, B_G-1), (A_2, B_G-2), ..., (A_G, B_1):
@@ -237,7 +237,8 @@ struct BufQueue {  // free TMEM buffers in the order they were handed over
 // (an integer conversion and a 64-bit add for every value of every chunk)
 // needs four warps a scheduler to keep up. Kernel alone, 4096 x 4096 x K
 // (group by group with eight epilogue warps -> this): K = 512 2.41 -> 1.58
-// ms, K = 2048 6.46 -> 5.46 ms, 400 clocks a K block where the MMAs take 256.
+// ms, K = 2048 6.46 -> 5.46 ms (5.54 with the magnitudes' product), 400 clocks
+// a K block where the MMAs take 256.
 template <int STAGES, bool PAIR>
 __global__ void __launch_bounds__(SLICE_THREADS, 1) slice_gemm_kernel(const __grid_constant__ SliceArgs P) {
   constexpr int A_BLK = BM * ROW_BYTES;  // one K block
